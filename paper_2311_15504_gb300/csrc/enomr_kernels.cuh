@@ -78,13 +78,13 @@ __device__ __forceinline__ void walk(const double *v, long long is0, int &sel, b
     }
 }
 
-// ENO-MR value of one window v[0..W-1] (v[g-1] = f_j).  All 32 lanes must
-// call it together; lanes with valid == false take part in the warp votes
-// only.  sA: shared copy of the a_l table of order R.
+// ENO-MR selection of one window v[0..W-1] (v[g-1] = f_j) in FP64.  All 32
+// lanes must call it together; lanes with valid == false take part in the
+// warp votes only.
 template <int R>
-__device__ __forceinline__ double mr_value(const double *v, const double *sA, bool valid, int &sel)
+__device__ __forceinline__ void mr_select(const double *v, bool valid, int &sel)
 {
-    constexpr int g = (R + 1) / 2, W = 2 * g - 1, T = Tab<R>::T, c = g - 1;
+    constexpr int g = (R + 1) / 2, T = Tab<R>::T, c = g - 1;
     // Step 1, Eq. (Baseline_IS)
     const double d1L = v[c] - v[c - 1];
     const double d2L = fma(-2.0, v[c - 1], v[c]) + v[c - 2];
@@ -98,21 +98,20 @@ __device__ __forceinline__ double mr_value(const double *v, const double *sA, bo
     walk<R, 0>(v, is0, sel, active);
     active = active || (valid && is0 == 0);
     // Step 3.2: minmod(a, b), a = f_{j+1} - f_j = -d1R, b = f_j - f_{j-1} = d1L
-    double mm = 0.0;
     if (active || !valid) {
         const long long ba = __double_as_longlong(d1R), bb = __double_as_longlong(d1L);
         const bool nz = abits(d1R) != 0 && abits(d1L) != 0;
         const bool same = nz && ((ba ^ bb) < 0);  // a = -d1R: signs of a, b agree
-        if (!same) {
-            sel = T + 2;
-        } else if (abits(d1R) <= abits(d1L)) {
-            sel = T;
-            mm = -d1R;
-        } else {
-            sel = T + 1;
-            mm = d1L;
-        }
+        sel = !same ? T + 2 : (abits(d1R) <= abits(d1L) ? T : T + 1);
     }
+}
+
+// Value of window v on the selection sel (0 .. T+2).  All 32 lanes call it
+// together.  sA: shared copy of the a_l table of order R.
+template <int R>
+__device__ __forceinline__ double mr_recon(const double *v, const double *sA, int sel)
+{
+    constexpr int g = (R + 1) / 2, W = 2 * g - 1, T = Tab<R>::T, c = g - 1;
     double val;
     if (__all_sync(FULL, sel == 0)) {
         val = Coef<R>::a(0) * v[0];
@@ -124,9 +123,20 @@ __device__ __forceinline__ double mr_value(const double *v, const double *sA, bo
 #pragma unroll
         for (int l = 0; l < W; ++l) val = fma(row[l], v[l], val);
     } else {
+        double mm = 0.0;
+        if (sel == T) mm = -(v[c] - v[c + 1]);
+        if (sel == T + 1) mm = v[c] - v[c - 1];
         val = fma(0.5, mm, v[c]);
     }
     return val;
+}
+
+// ENO-MR value of one window: selection, then value.
+template <int R>
+__device__ __forceinline__ double mr_value(const double *v, const double *sA, bool valid, int &sel)
+{
+    mr_select<R>(v, valid, sel);
+    return mr_recon<R>(v, sA, sel);
 }
 
 // Value of the ENO-MR reconstruction of window v with the choice given

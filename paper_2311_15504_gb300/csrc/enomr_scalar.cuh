@@ -3,9 +3,79 @@
 // One thread per interface; a CTA stages TP + 2g - 1 split flux values.
 #pragma once
 
-#include "enomr_kernels.cuh"
+#include "enomr_select.cuh"
 
 namespace enomr {
+
+// ENO-MR value of the window that starts at v0 and runs with stride DIRN (+1
+// or -1) through the split fluxes; e0: the pair of the difference of its
+// first two cells as stored (e[s] = f[s+1] - f[s]; a mirrored window meets
+// them in the opposite order and sign, which the caller's pointer and DIRN
+// express).  All 32 lanes of the warp call it together.  The FP64 pipe binds
+// these kernels: the selection runs in float (select_float), and a window on
+// a tested stencil whose differences are small against its centre takes the
+// float-pair sum; the others take the FP64 sums.  Measured (GB300, smooth data
+// with a square pulse): order 9, N = 1 048 573: 82 -> 34 us per launch, FP64
+// pipe 59 % busy; Burgers, order 13, N = 2^22: 387 -> 165 us.
+template <int R, int DIRN>
+__device__ __forceinline__ double scalar_value(const double *v0, const float2 *e0,
+                                               const double *sA, const float2 *sW, bool valid,
+                                               int &sel)
+{
+    constexpr int g = (R + 1) / 2, W = 2 * g - 1, T = Tab<R>::T, c = g - 1, N = W - 1;
+    using B = SelBound<2, 0>;
+    float e[N];
+    float emax = 0.0f;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        e[j] = e0[DIRN * j].x;
+        emax = fmaxf(emax, fabsf(e[j]));
+    }
+    const float vc = fabsf(to_float(v0[DIRN * c]));
+    const bool left0 = e[c - 1] == 0.0f && e[c - 2] == 0.0f;
+    const bool right0 = e[c] == 0.0f && e[c + 1] == 0.0f;
+    sel = select_float<R, B, false>(e, e, vc, left0, right0);
+    const bool open = valid && sel == SEL_OPEN;
+    if (__any_sync(FULL, open)) {
+        double v[W];
+#pragma unroll
+        for (int j = 0; j < W; ++j) v[j] = v0[DIRN * j];
+        int s64;
+        mr_select<R>(v, open, s64);
+        if (open) sel = s64;
+    }
+    // NaN differences do not enter emax: the float selection was open then
+    bool small = emax <= PAIR_RANGE * vc && sel < T;
+#pragma unroll
+    for (int j = 0; j < N; ++j) small = small && e[j] == e[j];
+    auto rest = [&](int j) { return DIRN > 0 ? e0[j] : make_float2(-e0[-j].x, -e0[-j].y); };
+    if (__all_sync(FULL, !valid || (small && sel == 0))) {
+        PairSum q;
+        q.first(Coef<R>::w()[0], rest(0));
+#pragma unroll
+        for (int j = 1; j < N; ++j) q.add(Coef<R>::w()[j], rest(j));
+        return v0[DIRN * c] + (widen(q.s) + widen(q.c));
+    }
+    if (__all_sync(FULL, !valid || small)) {
+        const float2 *w = sW + (valid ? sel : 0) * N;
+        PairSum q;
+        q.first(w[0], rest(0));
+#pragma unroll
+        for (int j = 1; j < N; ++j) q.add(w[j], rest(j));
+        return v0[DIRN * c] + (widen(q.s) + widen(q.c));
+    }
+    double v[W];
+#pragma unroll
+    for (int j = 0; j < W; ++j) v[j] = v0[DIRN * j];
+    return mr_recon<R>(v, sA, valid ? sel : 0);
+}
+
+template <int R>
+__device__ __forceinline__ void load_w_table(float2 *sW, int tid, int nthreads)
+{
+    constexpr int N = R - 1;
+    for (int i = tid; i < Tab<R>::T * N; i += nthreads) sW[i] = Coef<R>::w()[i];
+}
 
 // ---------------------------------------------------------------------------
 // Scalar advection f(u) = a u, alpha = |a|: f^+ = a u, f^- = 0 for a >= 0
@@ -16,25 +86,24 @@ __global__ void __launch_bounds__(TP) k_advection(AdvArgs A)
 {
     constexpr int g = (R + 1) / 2, W = 2 * g - 1, S = TP + 2 * g - 1, T = Tab<R>::T;
     __shared__ double sf[S];
+    __shared__ float2 se[S];  // e[s] = f[s+1] - f[s]
     __shared__ double sFh[TP];
     __shared__ double sA[T * W];
+    __shared__ float2 sW[T * (W - 1)];
     const int p = threadIdx.x;
     const long long x0 = (long long)blockIdx.x * (TP - 1);
     load_a_table<R>(sA, p, TP);
+    load_w_table<R>(sW, p, TP);
     for (int s = p; s < S; s += TP) sf[s] = A.a * A.U[ghost(x0 - g + s, A.n, A.bc)];
+    __syncthreads();
+    for (int s = p; s < S - 1; s += TP) se[s] = split_pair(sf[s + 1] - sf[s]);
     __syncthreads();
     const long long k = x0 + p;  // interface x_{k-1/2}
     const bool valid = k <= A.n;
-    double v[W];
-    if (A.a >= 0.0) {
-#pragma unroll
-        for (int j = 0; j < W; ++j) v[j] = sf[p + j];           // f^+ at cell k-1+l
-    } else {
-#pragma unroll
-        for (int j = 0; j < W; ++j) v[j] = sf[p + 2 * g - 1 - j];  // f^- at cell k-l
-    }
     int sel;
-    const double fh = mr_value<R>(v, sA, valid, sel);
+    const double fh = A.a >= 0.0 ? scalar_value<R, 1>(sf + p, se + p, sA, sW, valid, sel)
+                                 : scalar_value<R, -1>(sf + p + 2 * g - 1, se + p + 2 * g - 2, sA,
+                                                       sW, valid, sel);
     sFh[p] = fh;
     if (A.sel && valid) {
         const long long NI = A.n + 1;
@@ -67,11 +136,14 @@ __global__ void __launch_bounds__(TP) k_burgers(AdvArgs A)
     constexpr int g = (R + 1) / 2, W = 2 * g - 1, S = TP + 2 * g - 1, T = Tab<R>::T;
     __shared__ double sp[S];
     __shared__ double sm[S];
+    __shared__ float2 ep[S], em[S];  // differences of neighbouring split fluxes
     __shared__ double sFh[TP];
     __shared__ double sA[T * W];
+    __shared__ float2 sW[T * (W - 1)];
     const int p = threadIdx.x;
     const long long x0 = (long long)blockIdx.x * (TP - 1);
     load_a_table<R>(sA, p, TP);
+    load_w_table<R>(sW, p, TP);
     const double alpha = A.speed[0];
     const unsigned long long flags = (unsigned long long)__double_as_longlong(A.speed[1]);
     const int mode = !(flags & SGN_NEG) ? 0 : (!(flags & SGN_POS) ? 1 : 2);
@@ -94,21 +166,19 @@ __global__ void __launch_bounds__(TP) k_burgers(AdvArgs A)
         sm[s] = fm;
     }
     __syncthreads();
+    for (int s = p; s < S - 1; s += TP) {
+        if (mode != 1) ep[s] = split_pair(sp[s + 1] - sp[s]);
+        if (mode != 0) em[s] = split_pair(sm[s + 1] - sm[s]);
+    }
+    __syncthreads();
     const long long k = x0 + p;  // interface x_{k-1/2}
     const bool valid = k <= A.n;
-    double v[W];
     int selp = T + 2, selm = T + 2;
     double hp = 0.0, hm = 0.0;
-    if (mode != 1) {
-#pragma unroll
-        for (int j = 0; j < W; ++j) v[j] = sp[p + j];           // f^+ at cell k-1+l
-        hp = mr_value<R>(v, sA, valid, selp);
-    }
-    if (mode != 0) {
-#pragma unroll
-        for (int j = 0; j < W; ++j) v[j] = sm[p + 2 * g - 1 - j];  // f^- at cell k-l
-        hm = mr_value<R>(v, sA, valid, selm);
-    }
+    if (mode != 1)  // f^+ at cell k-1+l
+        hp = scalar_value<R, 1>(sp + p, ep + p, sA, sW, valid, selp);
+    if (mode != 0)  // f^- at cell k-l
+        hm = scalar_value<R, -1>(sm + p + 2 * g - 1, em + p + 2 * g - 2, sA, sW, valid, selm);
     sFh[p] = __dadd_rn(hp, hm);
     if (A.sel && valid) {
         A.sel[k] = (uint8_t)selp;

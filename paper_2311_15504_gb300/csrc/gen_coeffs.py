@@ -13,6 +13,21 @@ and the indicator of Eq. (CurrentIS), h^K P^(K) with K = m+n, is the
 
     b_s = sum_{i > s} (K+1)! / prod_{k != i} (xi_i - xi_k).
 
+Two further forms of the interface-value weights multiply the differences
+e_j = f_{j+1} - f_j of neighbouring cells instead of the cells.  As the a_l of a
+stencil add up to 1, sum_l a_l f_{c+l} = f_c + sum_j w_j e_j with
+
+    w_j = sum_{l > j} a_l  (j >= c),    w_j = -sum_{l <= j} a_l  (j < c),
+
+and with the full stencil on both sides of an interface (window a_l and its
+mirror image over 2g cells, middle pair g-1, g) the sum and the difference of
+the two reconstructions are
+
+    1/2 sum (a_j + a_{2g-1-j}) f_j = 1/2 (f_{g-1} + f_g) + sum_j s_j e_j,
+        sum (a_j - a_{2g-1-j}) f_j = sum_j d_j e_j.
+
+They are written as pairs of floats, high part (rounded to nearest) and rest.
+
 The candidate order is Eq. (Candidates); order R = 2r-1 keeps the entries
 with m, n <= r-1 and tests those with m, n >= 1 (Sec. 3.2, Step 3.1).
 
@@ -79,6 +94,45 @@ def hexlit(x: Fraction) -> str:
     return repr(v) if v.is_integer() else v.hex()
 
 
+def difference_weights(rowa, c: int):
+    """w_j, j = 0 .. W-2, of a window row (window centre c)."""
+    W = len(rowa)
+    return [(sum(rowa[j + 1:], Fraction(0)) if j >= c else -sum(rowa[:j + 1], Fraction(0)))
+            for j in range(W - 1)]
+
+
+def face_weights(rowa):
+    """s_j and d_j, j = 0 .. 2g-2, of the full window row."""
+    a = list(rowa) + [Fraction(0)]
+    n, g = len(a), len(a) // 2
+    t = [(a[j] + a[n - 1 - j]) / 2 - (Fraction(1, 2) if j in (g - 1, g) else 0) for j in range(n)]
+    d = [a[j] - a[n - 1 - j] for j in range(n)]
+    return [[-sum(v[:j + 1], Fraction(0)) for j in range(n - 1)] for v in (t, d)]
+
+
+def to_float(x: Fraction) -> Fraction:
+    """x rounded to 24 significant bits, to nearest even."""
+    if x == 0:
+        return x
+    e = math.floor(math.log2(abs(x)))
+    while Fraction(2) ** (e + 1) <= abs(x):
+        e += 1
+    while Fraction(2) ** e > abs(x):
+        e -= 1
+    q = Fraction(2) ** (e - 23)
+    return round(x / q) * q
+
+
+def pair(x: Fraction):
+    hi = to_float(x)
+    return hi, to_float(x - hi)
+
+
+def flit(x: Fraction) -> str:
+    v = float(x)
+    return "0.0f" if v == 0.0 else v.hex() + "f"
+
+
 def generate() -> str:
     out = []
     out.append("// Generated by gen_coeffs.py -- do not edit by hand.")
@@ -120,6 +174,13 @@ def generate() -> str:
         for row in as_:
             out.append("    " + ", ".join(hexlit(x) for x in row) + ",")
         out.append("};")
+        out.append("// {high, rest} of the difference weights w_j of every row, of s_j and of d_j")
+        for name, rows in ((f"kW{R}", [difference_weights(r, g - 1) for r in as_]),
+                           (f"kS{R}", face_weights(as_[0])[:1]), (f"kD{R}", face_weights(as_[0])[1:])):
+            out.append(f"static __constant__ float2 {name}[{sum(len(r) for r in rows)}] = {{")
+            for row in rows:
+                out.append("    " + ", ".join("{%s, %s}" % tuple(map(flit, pair(x))) for x in row) + ",")
+            out.append("};")
         out.append("")
     out.append("template <int R> struct Coef;")
     for R in ORDERS:
@@ -127,6 +188,8 @@ def generate() -> str:
         out.append(f"    __device__ static __forceinline__ double b(int i) {{ return kB{R}[i]; }}")
         out.append(f"    __device__ static __forceinline__ double a(int i) {{ return kA{R}[i]; }}")
         out.append(f"    __device__ static __forceinline__ const double *a_table() {{ return kA{R}; }}")
+        for f in "WSD":
+            out.append(f"    __device__ static __forceinline__ const float2 *{f.lower()}() {{ return k{f}{R}; }}")
         out.append("};")
     out.append("")
     out.append("}  // namespace enomr")
