@@ -50,6 +50,12 @@ struct enomr_ctx {
     // occupancy of the 2D sweeps: ENOMR_OCCUPANCY_AUTO / _HIGH / _LOW
     int occupancy;
     int sms;  // SMs of the device the context was created on
+    // block maps (TileMap) of U^n, U^(1) and U^(2), and the tile lists of the
+    // stage being evaluated
+    unsigned char *flat, *dead;  // [3][nby][nbx]
+    int *tile_lists;             // x tiles, y tiles, blocks
+    int *counts;                 // [6]
+    size_t zero_bytes;           // smax .. ay, cleared in one go
 };
 
 static void prof_start(enomr_ctx *c, int k)
@@ -103,6 +109,23 @@ __global__ void __launch_bounds__(256, 5) k_alpha(AlphaArgs A)
     const long long x = (long long)blockIdx.x * 32 + tx;
     const long long ty0 = (long long)blockIdx.y * 32, y0 = ty0 + 4 * ty;
     const long long ncell = A.nx * A.ny;
+    if (C == 4 && A.dead_a && blockIdx.x > 0 && blockIdx.y > 0) {
+        // This state was combined from two others.  Where this block and all
+        // around it are dead in both, they hold one state here too: no cell is
+        // a representative, and nothing is read.
+        bool dead = true;
+        if (tid < 9) {
+            const int bx = (int)blockIdx.x + tid % 3 - 1, by = (int)blockIdx.y + tid / 3 - 1;
+            if (bx < (int)gridDim.x && by < (int)gridDim.y) {
+                const long long b = (long long)by * gridDim.x + bx;
+                dead = A.dead_a[b] && A.dead_b[b];
+            }
+        }
+        if (__syncthreads_and(dead)) {
+            if (tid == 0) A.flat[(long long)blockIdx.y * gridDim.x + blockIdx.x] = 1;
+            return;
+        }
+    }
     if (tid < 96) {
         srow[tid / 3][tid % 3] = 0;
         scol[tid / 3][tid % 3] = 0;
@@ -137,6 +160,7 @@ __global__ void __launch_bounds__(256, 5) k_alpha(AlphaArgs A)
         for (int q = 0; q < C; ++q) ur[j][q] = valid ? A.U[q * ncell + y * A.nx + x] : 0.0;
     }
     __syncthreads();
+    bool differs = false;  // a cell here differs from its left or upper neighbour
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const long long y = y0 + j;
@@ -153,12 +177,14 @@ __global__ void __launch_bounds__(256, 5) k_alpha(AlphaArgs A)
             same_left = same_left && (__double_as_longlong(l) == __double_as_longlong(u[q]));
         }
         bool rep = valid && !same_left;
+        if (C == 4 && (tx > 0 || xl >= 0)) differs = differs || rep;
         if (C == 4) {
             bool same_up = j > 0 || have_up;
 #pragma unroll
             for (int q = 0; q < C; ++q)
                 same_up = same_up && (__double_as_longlong(up[q]) == __double_as_longlong(u[q]));
             rep = rep || (valid && !same_up);
+            if (j > 0 || have_up) differs = differs || (valid && !same_up);
 #pragma unroll
             for (int q = 0; q < C; ++q) up[q] = u[q];
         }
@@ -172,7 +198,12 @@ __global__ void __launch_bounds__(256, 5) k_alpha(AlphaArgs A)
                     (unsigned short)((4 * ty + j) * 32 + tx);
         }
     }
-    __syncthreads();
+    if (C == 4 && A.flat) {
+        const bool any = __syncthreads_or(differs) != 0;
+        if (tid == 0) A.flat[(long long)blockIdx.y * gridDim.x + blockIdx.x] = !any;
+    } else {
+        __syncthreads();
+    }
     const int n = nlist;
     if (n == 0) return;  // every cell repeats one outside the tile
     for (int b = ty * 32; b < n; b += 256) {
@@ -206,6 +237,85 @@ __global__ void __launch_bounds__(256, 5) k_alpha(AlphaArgs A)
             for (int k = 0; k < 3; ++k) atomicMax((unsigned long long *)(A.ay + 3 * x + k), scol[tid][k]);
     }
     if (tid == 0 && A.smax) atomicMax((unsigned long long *)A.smax, scfl);
+}
+
+// Dead blocks and tile lists of a state from its block flags (TileMap).  One
+// thread per block, then per x tile, then per y tile; each list is appended to
+// by whole warps.
+__global__ void __launch_bounds__(256) k_tile_map(TileMap m, unsigned nb256, unsigned nx256,
+                                                  unsigned ntx, unsigned nty, unsigned nsegx,
+                                                  unsigned ngrpy)
+{
+    const unsigned nb = (unsigned)m.nbx * m.nby;
+    auto dead = [&](int bx, int by) {
+        for (int dy = -1; dy <= 1; ++dy)
+            for (int dx = -1; dx <= 1; ++dx) {
+                const int x = bx + dx, y = by + dy;
+                if (x < 0 || y < 0 || x >= m.nbx || y >= m.nby) {
+                    if (m.closed) return false;
+                } else if (!m.flat[(long long)y * m.nbx + x]) {
+                    return false;
+                }
+            }
+        return true;
+    };
+    int *list, *count, item;
+    bool take = false;
+    if (blockIdx.x < nb256) {
+        const unsigned b = blockIdx.x * 256 + threadIdx.x;
+        list = m.blocks;
+        count = m.count + 2;
+        item = (int)b;
+        if (b < nb) {
+            take = dead((int)(b % m.nbx), (int)(b / m.nbx));
+            m.dead[b] = take;
+        }
+    } else if (blockIdx.x < nb256 + nx256) {
+        const unsigned t = (blockIdx.x - nb256) * 256 + threadIdx.x;
+        list = m.tiles_x;
+        count = m.count;
+        item = (int)t;
+        if (t < ntx) {
+            const long long x0 = (long long)(t % nsegx) * (X_TP - 1);
+            const long long x1 = x0 + X_TP - 2 < m.nx ? x0 + X_TP - 2 : m.nx - 1;
+            const int by = (int)((long long)(t / nsegx) * X_NL / MAP_B);
+            for (int bx = (int)(x0 / MAP_B); bx <= (int)(x1 / MAP_B) && !take; ++bx)
+                take = !dead(bx, by);
+        }
+    } else {
+        const unsigned t = (blockIdx.x - nb256 - nx256) * 256 + threadIdx.x;
+        list = m.tiles_y;
+        count = m.count + 1;
+        item = (int)t;
+        if (t < nty) {
+            const long long y0 = (long long)(t / ngrpy) * (Y_TP - 1);
+            const long long y1 = y0 + Y_TP - 2 < m.ny ? y0 + Y_TP - 2 : m.ny - 1;
+            const int bx = (int)((long long)(t % ngrpy) * Y_NL / MAP_B);
+            for (int by = (int)(y0 / MAP_B); by <= (int)(y1 / MAP_B) && !take; ++by)
+                take = !dead(bx, by);
+        }
+    }
+    const unsigned who = __ballot_sync(0xffffffffu, take);
+    if (who == 0) return;
+    const int lane = threadIdx.x & 31;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(count, __popc(who));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (take) list[base + __popc(who & ((1u << lane) - 1u))] = item;
+}
+
+cudaError_t launch_tile_map(const TileMap &m, cudaStream_t s)
+{
+    static_assert(MAP_B % X_NL == 0 && MAP_B % Y_NL == 0, "a tile's lines lie in one block");
+    const long long nb = (long long)m.nbx * m.nby;
+    const long long nsegx = (m.nx + X_TP - 2) / (X_TP - 1), ngrpx = (m.ny + X_NL - 1) / X_NL;
+    const long long nsegy = (m.ny + Y_TP - 2) / (Y_TP - 1), ngrpy = (m.nx + Y_NL - 1) / Y_NL;
+    const long long ntx = nsegx * ngrpx, nty = nsegy * ngrpy;
+    const long long b = (nb + 255) / 256, x = (ntx + 255) / 256, y = (nty + 255) / 256;
+    k_tile_map<<<(unsigned)(b + x + y), 256, 0, s>>>(m, (unsigned)b, (unsigned)x, (unsigned)ntx,
+                                                     (unsigned)nty, (unsigned)nsegx,
+                                                     (unsigned)ngrpy);
+    return cudaGetLastError();
 }
 
 // First cell (smallest index along its line) whose wave speed equals the
@@ -520,13 +630,37 @@ static enomr_status cu(cudaError_t e) { return e == cudaSuccess ? ENOMR_OK : ENO
 
 static int valid_order(int R) { return R >= 5 && R <= 17 && (R % 2) == 1; }
 
-// Per-line alpha of state U (zeroes the maxima first); smax on request.
-static enomr_status compute_alpha(enomr_ctx *c, const double *U, bool want_smax)
+// Block map slots: U^n, U^(1), U^(2) of a step; MAP_NONE: none is made.
+enum : int { MAP_NONE = -1, MAP_N = 0, MAP_1 = 1, MAP_2 = 2 };
+
+static long long map_blocks(const enomr_ctx *c)
+{
+    return ((c->nx + MAP_B - 1) / MAP_B) * ((c->ny + MAP_B - 1) / MAP_B);
+}
+
+// boundary sides or a body force: the 2D sweeps' EXT instances
+static bool extended(const enomr_ctx *c)
+{
+    return c->custom_sides || c->gx != 0.0 || c->gy != 0.0;
+}
+
+// Whether the 2D sweeps go by a block map: grids of at least 2^16 cells (a
+// smaller grid's sweeps end in the time that one more launch takes) with
+// 32-bit tile counts, without a body force (it changes dead blocks too).
+static bool map_allowed(const enomr_ctx *c)
+{
+    return c->ndim == 2 && c->flat && c->gx == 0.0 && c->gy == 0.0;
+}
+
+// Per-line alpha of state U (clears the maxima first); smax on request; map:
+// also the block flags, dead blocks and tile lists of U in that slot.  U^(1)
+// and U^(2) are combinations of the states of the slots before.
+static enomr_status compute_alpha(enomr_ctx *c, const double *U, bool want_smax,
+                                  int map = MAP_NONE)
 {
     if (c->eq == ENOMR_ADVECTION) return ENOMR_OK;
     if (c->eq == ENOMR_BURGERS) {
-        CU_TRY(cudaMemsetAsync(c->ax, 0, sizeof(double) * 2, c->stream));
-        if (want_smax) CU_TRY(cudaMemsetAsync(c->smax, 0, sizeof(double), c->stream));
+        CU_TRY(cudaMemsetAsync(c->smax, 0, (char *)(c->ax + 2) - (char *)c->smax, c->stream));
         prof_start(c, 3);
         cudaError_t e = launch_scalar_speed(U, c->nx, 1.0 / c->dx, c->ax,
                                             want_smax ? c->smax : nullptr, c->status, c->stream);
@@ -534,10 +668,10 @@ static enomr_status compute_alpha(enomr_ctx *c, const double *U, bool want_smax)
         return cu(e);
     }
     const int C = c->ndim == 2 ? 4 : 3;
-    CU_TRY(cudaMemsetAsync(c->ax, 0, sizeof(double) * 3 * c->ny, c->stream));
-    if (C == 4) CU_TRY(cudaMemsetAsync(c->ay, 0, sizeof(double) * 3 * c->nx, c->stream));
-    if (want_smax) CU_TRY(cudaMemsetAsync(c->smax, 0, sizeof(double), c->stream));
+    CU_TRY(cudaMemsetAsync(c->smax, 0, c->zero_bytes, c->stream));
+    const long long nb = map_blocks(c);
     AlphaArgs a;
+    memset(&a, 0, sizeof(a));
     a.U = U;
     a.nx = c->nx;
     a.ny = c->ny;
@@ -549,15 +683,39 @@ static enomr_status compute_alpha(enomr_ctx *c, const double *U, bool want_smax)
     a.ay = c->ay;
     a.smax = want_smax ? c->smax : nullptr;
     a.status = c->status;
+    if (map >= 0) {
+        a.flat = c->flat + map * nb;
+        if (map > 0) {
+            a.dead_a = c->dead;
+            a.dead_b = c->dead + (map - 1) * nb;
+        }
+    }
     prof_start(c, 3);
     cudaError_t e = launch_alpha(C, a, c->stream);
     prof_stop(c, 3);
+    if (e == cudaSuccess && map >= 0) {
+        TileMap m;
+        m.flat = a.flat;
+        m.dead = c->dead + map * nb;
+        m.nbx = (int)((c->nx + MAP_B - 1) / MAP_B);
+        m.nby = (int)((c->ny + MAP_B - 1) / MAP_B);
+        m.nx = c->nx;
+        m.ny = c->ny;
+        // a periodic line's ends, and sides, bring other states to the edges
+        m.closed = c->bc == ENOMR_PERIODIC || extended(c);
+        m.tiles_x = c->tile_lists;
+        m.tiles_y = m.tiles_x + ((c->nx + X_TP - 2) / (X_TP - 1)) * ((c->ny + X_NL - 1) / X_NL);
+        m.blocks = m.tiles_y + ((c->ny + Y_TP - 2) / (Y_TP - 1)) * ((c->nx + Y_NL - 1) / Y_NL);
+        m.count = c->counts;
+        e = launch_tile_map(m, c->stream);
+    }
     return cu(e);
 }
 
 static SweepArgs sweep_args(enomr_ctx *c, const double *U, bool ysweep)
 {
     SweepArgs a;
+    memset(&a, 0, sizeof(a));
     a.U = U;
     a.nx = c->nx;
     a.ny = c->ny;
@@ -586,30 +744,29 @@ static SweepArgs sweep_args(enomr_ctx *c, const double *U, bool ysweep)
     return a;
 }
 
-// boundary sides or a body force: the 2D sweeps' EXT instances
-static bool extended(const enomr_ctx *c)
-{
-    return c->custom_sides || c->gx != 0.0 || c->gy != 0.0;
-}
-
-// The 2D sweeps' low-occupancy instances: forced, or (automatic) for grids
-// whose x sweep has fewer tiles than four waves of the high-occupancy
-// instance.  Measured on GB300 (order 9): the paper's RP1 801^2 (3.7 waves),
-// double Mach reflection 1200x300 and Rayleigh-Taylor 200x800 whole runs
-// are 3-7 % faster with the low instance, the four-quadrant Riemann state at
-// 1024^2 (11 waves) and above is 30-40 % slower with it.
-static bool low_occupancy(const enomr_ctx *c)
+// The 2D sweeps' low-occupancy instances: forced, or (automatic) where a
+// launch lasts as long as a few tiles in sequence or its long path would
+// spill.  Over all tiles: grids whose x sweep has fewer tiles than four waves
+// of the high-occupancy instance.  Over a list, whose tiles are mostly ones
+// that a front crosses: from order 13 on (2048^2 Riemann state, order 17: 4.87
+// against 5.07 ms a step), and from order 9 on below eight waves (1024^2,
+// order 9: 1.05 against 1.18 ms; 2048^2: 2.06 against 1.91 ms); order 5 at
+// 801^2: 0.31 against 0.27 ms.
+static bool low_occupancy(const enomr_ctx *c, bool list)
 {
     if (c->occupancy == ENOMR_OCCUPANCY_LOW) return true;
     if (c->occupancy == ENOMR_OCCUPANCY_HIGH) return false;
     const long long tiles = ((c->nx + X_TP - 2) / (X_TP - 1)) * ((c->ny + X_NL - 1) / X_NL);
-    return tiles < 4LL * c->sms * (SWEEP_HIGH_THREADS_PER_SM / (X_TP * X_NL));
+    const long long wave = (long long)c->sms * (SWEEP_HIGH_THREADS_PER_SM / (X_TP * X_NL));
+    if (list) return c->order >= 13 || (c->order >= 9 && tiles < 8 * wave);
+    return tiles < 4 * wave;
 }
 
 // Evaluate L(U) into the epilogue.  The alpha of U must be current.
 static enomr_status rhs_with_epilogue(enomr_ctx *c, const double *U, const Epilogue &epi,
                                       uint8_t *sel, double *ft = nullptr, double t_coef = 0.0,
-                                      const uint8_t *sel_in = nullptr)
+                                      const uint8_t *sel_in = nullptr, int map = MAP_NONE,
+                                      bool un_mapped = false)
 {
     if (c->eq == ENOMR_ADVECTION || c->eq == ENOMR_BURGERS) {
         AdvArgs a;
@@ -642,15 +799,16 @@ static enomr_status rhs_with_epilogue(enomr_ctx *c, const double *U, const Epilo
     // results bit for bit); the EXT instances always load.
     const bool ext = extended(c);
     CUtensorMap mx, my;
-    const bool tma = !ext && c->staging != ENOMR_STAGING_LOADS && state_map(c, U, 0, &mx) &&
-                     state_map(c, U, 1, &my);
+    // Automatic staging: by TMA over all tiles, by loads over a list: its
+    // tiles differ in cost by more than ten, and the loading sweeps, one CTA
+    // per tile, spread them over the SMs better than the persistent ones
+    // (Riemann states, order 9, x / y sweep: 1024^2 167 / 167 us against
+    // 242 / 246, 2048^2 289 / 267 against 318 / 317).
+    const bool tma = !ext && (c->staging == ENOMR_STAGING_TMA ||
+                              (c->staging == ENOMR_STAGING_AUTO && map < 0)) &&
+                     state_map(c, U, 0, &mx) && state_map(c, U, 1, &my);
     if (c->staging == ENOMR_STAGING_TMA && !tma) return ENOMR_EINVAL;
-    const bool low = low_occupancy(c);
-    // Automatic staging: TMA for both sweeps wherever the state allows it
-    // (measured on GB300, 4096^2 Riemann state, orders 5-17: faster at every
-    // order in both directions, e.g. row sweep 0.35 against 0.39 ms and
-    // column sweep 0.75 against 0.81 ms at order 9, 0.58 against 0.74 and
-    // 1.17 against 1.35 ms at order 17).
+    const bool low = low_occupancy(c, map >= 0 && !ext);
     const bool tma_x = tma;
     const bool tma_y = tma;
     SweepArgs ax = sweep_args(c, U, false);
@@ -660,6 +818,12 @@ static enomr_status rhs_with_epilogue(enomr_ctx *c, const double *U, const Epilo
     ax.epi.mode = EPI_STORE;
     ax.epi.out = c->D;
     ax.t_coef = t_coef;
+    const long long nb = map_blocks(c);
+    if (map >= 0) {
+        ax.tiles = c->tile_lists;
+        ax.ntiles = c->counts;
+        ax.next = c->counts + 3;
+    }
     prof_start(c, 1);
     cudaError_t e = ext     ? by_order<E2XEF>(c->order, ax, low, c->stream)
                     : tma_x ? by_order<E2XTF>(c->order, mx, ax, low, c->stream)
@@ -673,6 +837,17 @@ static enomr_status rhs_with_epilogue(enomr_ctx *c, const double *U, const Epilo
     ay.epi = epi;
     ay.epi.Dprev = c->D;
     ay.t_coef = t_coef;
+    if (map >= 0) {
+        ay.tiles = c->tile_lists +
+                   ((c->nx + X_TP - 2) / (X_TP - 1)) * ((c->ny + X_NL - 1) / X_NL);
+        ay.ntiles = c->counts + 1;
+        ay.next = c->counts + 4;  // and [5]: dead blocks
+        ay.blocks = ay.tiles + ((c->ny + Y_TP - 2) / (Y_TP - 1)) * ((c->nx + Y_NL - 1) / Y_NL);
+        ay.nblocks = c->counts + 2;
+        ay.dead = c->dead + map * nb;
+        ay.un_dead = un_mapped ? c->dead : nullptr;
+        ay.nbx = (int)((c->nx + MAP_B - 1) / MAP_B);
+    }
     prof_start(c, 2);
     e = ext     ? by_order<E2YEF>(c->order, ay, low, c->stream)
         : tma_y ? by_order<E2YTF>(c->order, my, ay, low, c->stream)
@@ -708,9 +883,7 @@ ENOMR_API int enomr_num_tested(int R)
 ENOMR_API void enomr_free(enomr_ctx *c)
 {
     if (!c) return;
-    cudaFree(c->ax);
-    cudaFree(c->ay);
-    cudaFree(c->smax);
+    cudaFree(c->smax);  // with all that lies behind it
     cudaFree(c->dt);
     cudaFree(c->status);
     cudaFree(c->U1);
@@ -772,9 +945,16 @@ ENOMR_API enomr_status enomr_init(enomr_ctx **out, int eq, int ndim, int64_t nx,
     c->stream = (cudaStream_t)stream;
     const int C = eq != ENOMR_EULER ? 1 : (ndim == 2 ? 4 : 3);
     c->nstate = (long long)C * nx * ny;
-    bool ok = cudaMalloc(&c->ax, sizeof(double) * 3 * ny) == cudaSuccess &&
-              cudaMalloc(&c->ay, sizeof(double) * 3 * nx) == cudaSuccess &&
-              cudaMalloc(&c->smax, sizeof(double)) == cudaSuccess &&
+    // one block: smax, counts (6 ints), ax, ay (up to here cleared by one
+    // memset; in 1D without ay), then the tile lists and the block maps
+    const size_t zero_all = sizeof(double) * (4 + 3 * (size_t)ny + 3 * (size_t)nx);
+    c->zero_bytes = ndim == 2 ? zero_all : sizeof(double) * (4 + 3 * (size_t)ny);
+    const long long nb = map_blocks(c);
+    const long long lists = ((nx + X_TP - 2) / (X_TP - 1)) * ((ny + X_NL - 1) / X_NL) +
+                            ((ny + Y_TP - 2) / (Y_TP - 1)) * ((nx + Y_NL - 1) / Y_NL) + nb;
+    const bool mapped = ndim == 2 && nx * ny >= (1LL << 16) && lists < (1LL << 30);
+    const size_t map_bytes = mapped ? sizeof(int) * lists + 6 * nb : 0;
+    bool ok = cudaMalloc(&c->smax, zero_all + map_bytes) == cudaSuccess &&
               cudaMalloc(&c->dt, sizeof(double)) == cudaSuccess &&
               cudaMalloc(&c->status, sizeof(int)) == cudaSuccess &&
               cudaMalloc(&c->U1, sizeof(double) * c->nstate) == cudaSuccess &&
@@ -794,6 +974,16 @@ ENOMR_API enomr_status enomr_init(enomr_ctx **out, int eq, int ndim, int64_t nx,
         for (int i = 0; i < 2 && ok; ++i)
             ok = cudaMalloc(&c->fsel[i], c->nsel) == cudaSuccess &&
                  cudaMalloc(&c->fft[i], sizeof(double) * c->nft) == cudaSuccess;
+    }
+    if (ok) {
+        c->counts = (int *)(c->smax + 1);
+        c->ax = c->smax + 4;
+        c->ay = c->ax + 3 * ny;
+        if (mapped) {
+            c->tile_lists = (int *)(c->ay + 3 * nx);
+            c->flat = (unsigned char *)(c->tile_lists + lists);
+            c->dead = c->flat + 3 * nb;
+        }
     }
     if (!ok) {
         cudaGetLastError();
@@ -829,23 +1019,28 @@ ENOMR_API enomr_status enomr_set_stream(enomr_ctx *c, void *stream)
 ENOMR_API enomr_status enomr_rhs(enomr_ctx *c, const double *U, double *dUdt)
 {
     if (!c || !U || !dUdt || (const double *)dUdt == U) return ENOMR_EINVAL;
-    enomr_status st = compute_alpha(c, U, false);
+    const int map = map_allowed(c) ? MAP_N : MAP_NONE;
+    enomr_status st = compute_alpha(c, U, false, map);
     if (st) return st;
     Epilogue e;
     memset(&e, 0, sizeof(e));
     e.mode = EPI_STORE;
     e.out = dUdt;
-    return rhs_with_epilogue(c, U, e, nullptr);
+    return rhs_with_epilogue(c, U, e, nullptr, nullptr, 0.0, nullptr, map);
 }
 
 static const double RK_C0[3] = {0.0, 0.75, 1.0 / 3.0};
 static const double RK_C1[3] = {1.0, 0.25, 2.0 / 3.0};
 
+// step: stage s of a step whose stages run one after another, so that the
+// block maps of U^n and of the stage before hold (slot s - 1 is this one's).
 static enomr_status stage_impl(enomr_ctx *c, int s, const double *Un, const double *Us,
                                double *Uout, bool alpha_current = false, uint8_t *sel = nullptr,
-                               double *ft = nullptr)
+                               double *ft = nullptr, bool step = false)
 {
-    enomr_status st = alpha_current ? ENOMR_OK : compute_alpha(c, Us, false);
+    // recorded selections and values need every interface evaluated
+    const int map = sel || ft || !map_allowed(c) ? MAP_NONE : (step ? s - 1 : MAP_N);
+    enomr_status st = alpha_current ? ENOMR_OK : compute_alpha(c, Us, false, map);
     if (st) return st;
     Epilogue e;
     memset(&e, 0, sizeof(e));
@@ -856,7 +1051,7 @@ static enomr_status stage_impl(enomr_ctx *c, int s, const double *Un, const doub
     e.Un = Un;
     e.out = Uout;
     static const double RK_T[3] = {0.0, 1.0, 0.5};  // stage times t + RK_T dt
-    return rhs_with_epilogue(c, Us, e, sel, ft, RK_T[s - 1]);
+    return rhs_with_epilogue(c, Us, e, sel, ft, RK_T[s - 1], nullptr, map, step);
 }
 
 ENOMR_API enomr_status enomr_stage(enomr_ctx *c, int s, const double *Un, const double *Us,
@@ -870,7 +1065,8 @@ ENOMR_API enomr_status enomr_stage(enomr_ctx *c, int s, const double *Un, const 
     return stage_impl(c, s, Un, Us, Uout);
 }
 
-static enomr_status set_step_dt(enomr_ctx *c, const double *U, double dt, double cfl)
+static enomr_status set_step_dt(enomr_ctx *c, const double *U, double dt, double cfl,
+                                int map = MAP_NONE)
 {
     if (dt > 0.0) return cu(launch_set_dt(c->smax, 0.0, dt, c->dt, c->stream));
     if (!(cfl > 0.0)) return ENOMR_EINVAL;
@@ -878,7 +1074,7 @@ static enomr_status set_step_dt(enomr_ctx *c, const double *U, double dt, double
         if (!(c->adv != 0.0)) return ENOMR_EINVAL;
         return cu(launch_set_dt(c->smax, 0.0, cfl * c->dx / fabs(c->adv), c->dt, c->stream));
     }
-    enomr_status st = compute_alpha(c, U, true);
+    enomr_status st = compute_alpha(c, U, true, map);
     if (st) return st;
     return cu(launch_set_dt(c->smax, cfl, 0.0, c->dt, c->stream));
 }
@@ -886,13 +1082,13 @@ static enomr_status set_step_dt(enomr_ctx *c, const double *U, double dt, double
 ENOMR_API enomr_status enomr_step(enomr_ctx *c, double *U, double dt, double cfl, double *dt_used)
 {
     if (!c || !U) return ENOMR_EINVAL;
-    enomr_status st = set_step_dt(c, U, dt, cfl);
+    enomr_status st = set_step_dt(c, U, dt, cfl, map_allowed(c) ? MAP_N : MAP_NONE);
     if (st) return st;
     // with a CFL step the alpha of U^n was just computed with the wave-speed max
     const bool alpha_done = !(dt > 0.0) && c->eq != ENOMR_ADVECTION;
-    if ((st = stage_impl(c, 1, U, U, c->U1, alpha_done))) return st;
-    if ((st = stage_impl(c, 2, U, c->U1, c->U2))) return st;
-    if ((st = stage_impl(c, 3, U, c->U2, U))) return st;
+    if ((st = stage_impl(c, 1, U, U, c->U1, alpha_done, nullptr, nullptr, true))) return st;
+    if ((st = stage_impl(c, 2, U, c->U1, c->U2, false, nullptr, nullptr, true))) return st;
+    if ((st = stage_impl(c, 3, U, c->U2, U, false, nullptr, nullptr, true))) return st;
     if (extended(c)) {  // the time only matters to boundary sides
         k_advance_time<<<1, 1, 0, c->stream>>>(c->t_dev, c->dt, 1.0);
         CU_TRY(cudaGetLastError());

@@ -48,6 +48,23 @@ struct SideDev {
     double st_lo[4], st_hi[4];
 };
 
+// Map of the cell blocks of a 2D state that hold one state together with all
+// the blocks around them ("dead" blocks: every flux difference of their cells
+// is exactly zero), and the lists made from it: the tiles of both sweeps that
+// touch another block, and the dead blocks.
+constexpr int MAP_B = 32;  // cells per block side; at least the widest halo, 9
+struct TileMap {
+    const unsigned char *flat;  // [nby][nbx]: every cell equals its left and upper neighbour
+    unsigned char *dead;        // [nby][nbx]
+    int nbx, nby;
+    long long nx, ny;
+    int closed;                 // blocks at the edges of the domain are never dead
+    int *tiles_x, *tiles_y, *blocks;
+    int *count;                 // [3], zeroed before the launch: x tiles, y tiles, dead blocks
+                                // ([3..5]: SweepArgs::next of the two sweeps, dead blocks taken)
+};
+cudaError_t launch_tile_map(const TileMap &m, cudaStream_t s);
+
 // One 1D line sweep of the Euler equations (1D: C = 3; 2D x or y sweep: C = 4).
 struct SweepArgs {
     const double *U;       // stage state, [C][ny][nx]
@@ -73,6 +90,14 @@ struct SweepArgs {
     // body force in line components (normal, tangential); applied when src
     int src;
     double g_n, g_t;
+    // 2D sweeps over the tiles of a list (TileMap); null: over all tiles.  The
+    // column sweep leaves the cells of dead blocks to write_dead_block, which
+    // fills the blocks of a second list; un_dead (optional): blocks that are
+    // dead in epi.Un too
+    const int *tiles, *ntiles, *blocks, *nblocks;
+    int *next;  // zeroed before the launch: entries handed out beyond one per CTA (TMA sweeps)
+    const unsigned char *dead, *un_dead;
+    int nbx;
 };
 
 struct AdvArgs {
@@ -93,6 +118,10 @@ struct AlphaArgs {
     double *ay;            // [nx][3] (2D only), zeroed before the launch
     double *smax;          // CFL wave-speed max (may be nullptr)
     int *status;
+    // optional (2D): block flags of this state (TileMap::flat), and the dead
+    // blocks of the two states it was combined from
+    unsigned char *flat;
+    const unsigned char *dead_a, *dead_b;
 };
 
 // Batched 1D Euler (problem-major packing: problem p's [3][n_p] block starts

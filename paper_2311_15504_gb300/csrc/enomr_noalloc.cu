@@ -111,6 +111,7 @@ extern "C" ENOMR_API enomr_status enomr_rhs_euler2d_noalloc(const double *U, dou
         return ENOMR_ECUDA;
 
     enomr::AlphaArgs aa;
+    memset(&aa, 0, sizeof(aa));
     aa.U = U;
     aa.nx = nx;
     aa.ny = ny;

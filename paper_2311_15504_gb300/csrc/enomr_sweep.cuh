@@ -717,7 +717,10 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs &A, long long x0, lon
     unsigned long long ws[3] = {0, 0, 0};
     if (p < TP - 1 && Lg < nlines) {
         const long long i = x0 + p;
-        if (i < nlen) {
+        // cells of dead blocks are written by write_dead_block
+        const bool mine = DIR == 0 || C != 4 || !A.dead ||
+                          !A.dead[(i / MAP_B) * A.nbx + Lg / MAP_B];
+        if (i < nlen && mine) {
             const long long gi = (DIR == 0) ? Lg * nx + i : i * nx + Lg;
             const int sc = p + g;  // staged index of cell i
             double o[C];
@@ -786,6 +789,53 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs &A, long long x0, lon
     }
 }
 
+// The cells of dead block b (TileMap): one state, whose flux differences are
+// exactly zero in both directions, so D = -0 as the sweeps store it.  All 256
+// threads; each warp evaluates the combination of the block's state once and
+// stores it to its 4 rows of 32 cells, without reading U beyond one cell; Un
+// is read cell by cell unless it is known to be one state too.  Bound by the
+// store bandwidth, and by the reads of Un where they are needed.
+inline constexpr int DEAD_THREADS = 256;
+__device__ __forceinline__ void write_dead_block(const SweepArgs &A, int b)
+{
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const long long nx = A.nx, ny = A.ny, ncell = nx * ny;
+    const int by = b / A.nbx, bx = b - by * A.nbx;
+    const long long x = (long long)bx * MAP_B + tx, y0 = (long long)by * MAP_B;
+    const long long first = y0 * nx + (long long)bx * MAP_B;
+    const Epilogue &e = A.epi;
+    const bool stage = e.mode == EPI_STAGE && !(e.c0 == 0.0 && e.c1 == 1.0);
+    auto combine = [&](double un, double us) {
+        if (e.mode == EPI_STORE) return -0.0;
+        const double w = fma(*e.dt_dev, -0.0, us);
+        return stage ? fma(e.c0, un, e.c1 * w) : w;
+    };
+    // lane q: component q
+    const int ql = tx & 3;
+    const double us = A.U[ql * ncell + first], un = stage ? e.Un[ql * ncell + first] : 0.0;
+    const double r = combine(un, us);
+    const bool read = stage && !(A.un_dead && A.un_dead[b]);
+    __syncthreads();  // out may be Un: every warp has the first cell before any stores
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const double rq = __shfl_sync(FULL, r, q), uq = __shfl_sync(FULL, un, q),
+                     sq = __shfl_sync(FULL, us, q);
+#pragma unroll
+        for (int j = 0; j < MAP_B / 8; ++j) {
+            const long long y = y0 + ty * (MAP_B / 8) + j;
+            if (x < nx && y < ny) {
+                const long long i = q * ncell + y * nx + x;
+                double o = rq;
+                if (read) {
+                    const double u = e.Un[i];
+                    if (__double_as_longlong(u) != __double_as_longlong(uq)) o = combine(u, sq);
+                }
+                e.out[i] = o;
+            }
+        }
+    }
+}
+
 // Resident sweep threads per SM: 1280 (40 warps, five 256-thread CTAs,
 // which is also what the shared memory of the 2D tiles allows) caps the
 // registers at 48.  The flat interfaces, most of a typical grid, need few
@@ -816,9 +866,25 @@ __global__ void __launch_bounds__(TP *NL, MINB) k_sweep(SweepArgs A)
     constexpr int g = (R + 1) / 2, W = 2 * g - 1, T = Tab<R>::T;
     __shared__ SweepSmem<R, C, TP, NL> sm;
     __shared__ double sA[T * W];
+    unsigned seg = (DIR == 0) ? blockIdx.x : blockIdx.y, grp = (DIR == 0) ? blockIdx.y : blockIdx.x;
+    if constexpr (C == 4) {
+        if (A.tiles) {
+            // this CTA's tile is an entry of the list; the dead blocks go to
+            // the CTAs past its end first
+            const unsigned id = blockIdx.y * gridDim.x + blockIdx.x, n = (unsigned)*A.ntiles;
+            if constexpr (DIR == 1) {
+                const unsigned all = gridDim.x * gridDim.y, nblk = (unsigned)*A.nblocks;
+                for (unsigned b = all - 1 - id; b < nblk; b += all) write_dead_block(A, A.blocks[b]);
+            }
+            if (id >= n) return;
+            const unsigned t = (unsigned)A.tiles[id], q = t / gridDim.x, r = t - q * gridDim.x;
+            seg = (DIR == 0) ? r : q;
+            grp = (DIR == 0) ? q : r;
+        }
+    }
     load_a_table<R>(sA, threadIdx.x, TP * NL);
-    const long long x0 = (long long)((DIR == 0) ? blockIdx.x : blockIdx.y) * (TP - 1);
-    const long long l0 = (long long)((DIR == 0) ? blockIdx.y : blockIdx.x) * NL;
+    const long long x0 = (long long)seg * (TP - 1);
+    const long long l0 = (long long)grp * NL;
     sweep_tile<R, C, DIR, TP, NL, EXT, LM>(A, x0, l0, sA, ClassicTile<R, C, DIR, TP, NL>{sm});
 }
 

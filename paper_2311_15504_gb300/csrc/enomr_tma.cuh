@@ -51,6 +51,8 @@ struct TmaSmem {
     };
     double sA[T * W];
     unsigned long long full[2];  // mbarriers of the ring slots
+    long long next;              // the CTA's next list entry and its tile
+    unsigned next_tile;
     int nlist;
     int nrep;
 };
@@ -193,7 +195,7 @@ struct TmaGeom {
 // processed tiles of a wave share DRAM pages).
 template <int R, int DIR, int TP, int NL, int MINB, bool SP>
 __global__ void __launch_bounds__(TP *NL, MINB)
-    k_sweep_tma(const __grid_constant__ CUtensorMap map, SweepArgs A, long long ntiles)
+    k_sweep_tma(const __grid_constant__ CUtensorMap map, SweepArgs A, long long ntiles_all)
 {
     constexpr int C = 4;
     using SM = TmaSmem<R, C, DIR, TP, NL, SP>;
@@ -212,13 +214,17 @@ __global__ void __launch_bounds__(TP *NL, MINB)
     // tile count below 2^31, so 32-bit division suffices (64-bit division is
     // a long software sequence)
     const unsigned nfast = (unsigned)((DIR == 0) ? nseg : ngrp);
-    auto tile_of = [&](long long t, long long &x0, long long &l0) {
-        const unsigned tt = (unsigned)t, q = tt / nfast, r = tt - q * nfast;
+    const long long ntiles = A.tiles ? (long long)*A.ntiles : ntiles_all;
+    auto index = [&](long long t) {
+        return t >= ntiles ? 0u : (A.tiles ? (unsigned)A.tiles[t] : (unsigned)t);
+    };
+    auto tile_of = [&](unsigned tt, long long &x0, long long &l0) {
+        const unsigned q = tt / nfast, r = tt - q * nfast;
         const unsigned seg = (DIR == 0) ? r : q, grp = (DIR == 0) ? q : r;
         x0 = (long long)seg * (TP - 1);
         l0 = (long long)grp * NL;
     };
-    auto issue = [&](long long t, int slot) {
+    auto issue = [&](unsigned t, int slot) {
         long long x0, l0;
         tile_of(t, x0, l0);
         mbar_expect_tx(&sm.full[slot], BYTES);
@@ -238,17 +244,28 @@ __global__ void __launch_bounds__(TP *NL, MINB)
     }
     load_a_table<R>(sm.sA, tid, NT);
     __syncthreads();
-    if (tid == 0 && (long long)blockIdx.x < ntiles) issue(blockIdx.x, 0);
+    // Tiles: in a list the cost of a tile varies by more than ten (a front
+    // crosses it or not), so entries beyond the first of each CTA are handed
+    // out as the CTAs get to them; over all tiles the order is fixed.  Thread
+    // 0 takes the next entry a tile ahead, and the barrier that follows its
+    // copy's issue passes it on.
+    long long t = blockIdx.x;
+    unsigned cur = index(t);
+    if (tid == 0 && t < ntiles) issue(cur, 0);
 
-    int it = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++it) {
+    for (int it = 0; t < ntiles; ++it) {
         const int slot = it & 1;
-        const long long tn = t + gridDim.x;
-        if (tid == 0 && tn < ntiles) {
-            // the other slot was released by the barrier that ended the
-            // previous tile; order its generic-proxy accesses before the copy
-            fence_proxy_async();
-            issue(tn, slot ^ 1);
+        if (tid == 0) {
+            const long long tn =
+                A.tiles ? (long long)gridDim.x + atomicAdd(A.next, 1) : t + gridDim.x;
+            sm.next = tn;
+            sm.next_tile = index(tn);
+            if (tn < ntiles) {
+                // the other slot was released by the barrier that ended the
+                // previous tile; order its generic-proxy accesses before the copy
+                fence_proxy_async();
+                issue(sm.next_tile, slot ^ 1);
+            }
         }
         const bool ok = mbar_wait(&sm.full[slot], (unsigned)((it >> 1) & 1), TMA_WAIT_LIMIT);
         if (__syncthreads_or(!ok)) {
@@ -256,13 +273,15 @@ __global__ void __launch_bounds__(TP *NL, MINB)
             // in flight into the other slot, and stop
             if (tid == 0) {
                 atomicOr(A.status, ST_TMA_TIMEOUT);
-                if (tn < ntiles) mbar_wait(&sm.full[slot ^ 1], (unsigned)(((it + 1) >> 1) & 1),
+                if (sm.next < ntiles) mbar_wait(&sm.full[slot ^ 1], (unsigned)(((it + 1) >> 1) & 1),
                                            TMA_WAIT_LIMIT);
             }
             return;
         }
         long long x0, l0;
-        tile_of(t, x0, l0);
+        tile_of(cur, x0, l0);
+        t = sm.next;
+        cur = sm.next_tile;
         double *base = sm.raw[slot];
         if (DIR == 0) base += (x0 - g) & 1;  // the copy started at the even x at or below x0 - g
         const TmaTile<R, C, DIR, TP, NL, SP> tile{sm, base};
@@ -292,6 +311,21 @@ __global__ void __launch_bounds__(TP *NL, MINB)
         }
         sweep_tile<R, C, DIR, TP, NL, false>(A, x0, l0, sm.sA, tile);
         __syncthreads();  // the slot and the tile arrays are free again
+    }
+    if constexpr (DIR == 1) {
+        static_assert(NT == DEAD_THREADS, "write_dead_block works with 256 threads");
+        if (A.tiles) {
+            // dead blocks, four at a time, as the CTAs run out of tiles
+            const int n = *A.nblocks;
+            for (;;) {
+                if (tid == 0) sm.next = atomicAdd(A.next + 1, 4);
+                __syncthreads();
+                const int b0 = (int)sm.next;
+                __syncthreads();
+                if (b0 >= n) break;
+                for (int b = b0; b < b0 + 4 && b < n; ++b) write_dead_block(A, A.blocks[b]);
+            }
+        }
     }
 }
 
