@@ -744,22 +744,18 @@ static SweepArgs sweep_args(enomr_ctx *c, const double *U, bool ysweep)
     return a;
 }
 
-// The 2D sweeps' low-occupancy instances: forced, or (automatic) where a
-// launch lasts as long as a few tiles in sequence or its long path would
-// spill.  Over all tiles: grids whose x sweep has fewer tiles than four waves
-// of the high-occupancy instance.  Over a list, whose tiles are mostly ones
-// that a front crosses: from order 13 on (2048^2 Riemann state, order 17: 4.87
-// against 5.07 ms a step), and from order 9 on below eight waves (1024^2,
-// order 9: 1.05 against 1.18 ms; 2048^2: 2.06 against 1.91 ms); order 5 at
-// 801^2: 0.31 against 0.27 ms.
+// The 2D sweeps' low-occupancy instances: forced, or (automatic) over all
+// tiles of grids whose x sweep has fewer tiles than four waves of the
+// high-occupancy instance, whose launches last as long as a few tiles in
+// sequence.  Over a list the high-occupancy instance (Riemann states, a step:
+// 801^2 order 5 0.26 against 0.30 ms, 1024^2 order 9 0.96 / 1.02, 2048^2
+// order 13 2.33 / 2.81, order 17 3.66 / 4.42, 4096^2 order 9 3.01 / 4.18).
 static bool low_occupancy(const enomr_ctx *c, bool list)
 {
     if (c->occupancy == ENOMR_OCCUPANCY_LOW) return true;
-    if (c->occupancy == ENOMR_OCCUPANCY_HIGH) return false;
+    if (c->occupancy == ENOMR_OCCUPANCY_HIGH || list) return false;
     const long long tiles = ((c->nx + X_TP - 2) / (X_TP - 1)) * ((c->ny + X_NL - 1) / X_NL);
-    const long long wave = (long long)c->sms * (SWEEP_HIGH_THREADS_PER_SM / (X_TP * X_NL));
-    if (list) return c->order >= 13 || (c->order >= 9 && tiles < 8 * wave);
-    return tiles < 4 * wave;
+    return tiles < 4LL * c->sms * (SWEEP_HIGH_THREADS_PER_SM / (X_TP * X_NL));
 }
 
 // Evaluate L(U) into the epilogue.  The alpha of U must be current.

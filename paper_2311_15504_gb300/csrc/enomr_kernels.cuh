@@ -25,6 +25,7 @@
 
 #include "enomr_coeffs.h"
 #include "enomr_common.cuh"
+#include "enomr_float.cuh"
 #include "enomr_internal.h"
 
 namespace enomr {
@@ -82,7 +83,7 @@ __device__ __forceinline__ void walk(const double *v, long long is0, int &sel, b
 // lanes must call it together; lanes with valid == false take part in the
 // warp votes only.
 template <int R>
-__device__ __forceinline__ void mr_select(const double *v, bool valid, int &sel)
+__device__ __forceinline__ void mr_select64(const double *v, bool valid, int &sel)
 {
     constexpr int g = (R + 1) / 2, T = Tab<R>::T, c = g - 1;
     // Step 1, Eq. (Baseline_IS)
@@ -103,6 +104,79 @@ __device__ __forceinline__ void mr_select(const double *v, bool valid, int &sel)
         const bool nz = abits(d1R) != 0 && abits(d1L) != 0;
         const bool same = nz && ((ba ^ bb) < 0);  // a = -d1R: signs of a, b agree
         sel = !same ? T + 2 : (abits(d1R) <= abits(d1L) ? T : T + 1);
+    }
+}
+
+// The same selection from the differences e_j = v_{j+1} - v_j in float, each
+// comparison with a bound on its distance from the FP64 values' (SelBound);
+// windows that it leaves open are selected in FP64, so the outcome is that of
+// mr_select64 always.  FP64 work: 2g - 2 subtractions instead of 6 + m + n + 1
+// operations for every candidate that is tested (10 to 26 of them at a front,
+// orders 9 to 17); the FP32 pipe does 64 operations in the time of one of
+// those.  The walk is a loop over the coefficient table (constant operands,
+// one candidate at a time for the whole warp) to keep the code small: the
+// sweeps hold several copies of it.
+template <int R>
+__device__ __forceinline__ void mr_select(const double *v, bool valid, int &sel)
+{
+    constexpr int g = (R + 1) / 2, T = Tab<R>::T, c = g - 1, N = 2 * g - 2;
+    using B = SelBound<2, 0>;
+    float e[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) e[j] = to_float(v[j + 1] - v[j]);
+    const float S = fabsf(to_float(v[c]));
+    const bool none = (e[c - 1] == 0.0f && e[c - 2] == 0.0f) || (e[c] == 0.0f && e[c + 1] == 0.0f);
+    const float al = fabsf(e[c - 1]), ar = fabsf(e[c]), sv = S * B::values(2);
+    const float el = __fmaf_rn(al + fabsf(e[c - 2]), B::terms(2), sv);
+    const float er = __fmaf_rn(ar + fabsf(e[c + 1]), B::terms(2), sv);
+    const float L = fmaxf(al, fabsf(e[c - 1] - e[c - 2])), Q = fmaxf(ar, fabsf(e[c + 1] - e[c]));
+    const float lo = fminf(L - el, Q - er), hi = fminf(L + el, Q + er);
+    bool open = !(S <= 0x1p90f) || !(el + er <= 0x1p90f);  // NaN, out of range
+    sel = valid ? T : 0;
+    bool active = valid && !none && !open;
+#pragma unroll 1
+    for (int t = 0; t < T && __any_sync(FULL, active); ++t) {
+        float s = 0.0f, a = 0.0f;
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const float b = Coef<R>::e()[t * N + j];
+            s = __fmaf_rn(b, e[j], s);
+            a = __fmaf_rn(fabsf(b), fabsf(e[j]), a);
+        }
+        const int K = Coef<R>::order(t);
+        const float err = __fmaf_rn(a, 0x1p-24f * (float)(K + 4),
+                                    S * (B::values(0) * __int_as_float((127 + K) << 23)));
+        s = fabsf(s);
+        if (active && s + err < lo) {
+            sel = t;
+            active = false;
+        } else if (active && !(s - err > hi)) {
+            open = true;
+            active = false;
+        }
+    }
+    if (none) {
+        if (valid) sel = T + 2;  // IS_0 = 0: no candidate passes, minmod(a, b) = 0
+        open = false;
+    } else if (active) {
+        // minmod(f_{j+1} - f_j, f_j - f_{j-1})
+        const float e1 = __fmaf_rn(al, B::terms(2), sv), e2 = __fmaf_rn(ar, B::terms(2), sv);
+        if (!(al > e1) || !(ar > e2))
+            open = true;
+        else if ((e[c - 1] < 0.0f) != (e[c] < 0.0f))
+            sel = T + 2;
+        else if (ar + e2 < al - e1)
+            sel = T;
+        else if (al + e1 < ar - e2)
+            sel = T + 1;
+        else
+            open = true;
+    }
+    open = open && valid;
+    if (__any_sync(FULL, open)) {
+        int s64;
+        mr_select64<R>(v, open, s64);
+        if (open) sel = s64;
     }
 }
 

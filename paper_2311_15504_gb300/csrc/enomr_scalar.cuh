@@ -41,33 +41,39 @@ __device__ __forceinline__ double scalar_value(const double *v0, const float2 *e
 #pragma unroll
         for (int j = 0; j < W; ++j) v[j] = v0[DIRN * j];
         int s64;
-        mr_select<R>(v, open, s64);
+        mr_select64<R>(v, open, s64);
         if (open) sel = s64;
     }
     // NaN differences do not enter emax: the float selection was open then
-    bool small = emax <= PAIR_RANGE * vc && sel < T;
+    bool small = emax <= PAIR_RANGE * vc && sel < T && valid;
 #pragma unroll
     for (int j = 0; j < N; ++j) small = small && e[j] == e[j];
+    // the form is each lane's own choice: the face shared by two tiles takes
+    // the same one in both
     auto rest = [&](int j) { return DIRN > 0 ? e0[j] : make_float2(-e0[-j].x, -e0[-j].y); };
-    if (__all_sync(FULL, !valid || (small && sel == 0))) {
+    double value = 0.0;
+    if (__all_sync(FULL, !small || sel == 0)) {
         PairSum q;
         q.first(Coef<R>::w()[0], rest(0));
 #pragma unroll
         for (int j = 1; j < N; ++j) q.add(Coef<R>::w()[j], rest(j));
-        return v0[DIRN * c] + (widen(q.s) + widen(q.c));
-    }
-    if (__all_sync(FULL, !valid || small)) {
-        const float2 *w = sW + (valid ? sel : 0) * N;
+        value = v0[DIRN * c] + (widen(q.s) + widen(q.c));
+    } else if (small) {
+        const float2 *w = sW + sel * N;
         PairSum q;
         q.first(w[0], rest(0));
 #pragma unroll
         for (int j = 1; j < N; ++j) q.add(w[j], rest(j));
-        return v0[DIRN * c] + (widen(q.s) + widen(q.c));
+        value = v0[DIRN * c] + (widen(q.s) + widen(q.c));
     }
-    double v[W];
+    if (__any_sync(FULL, valid && !small)) {
+        double v[W];
 #pragma unroll
-    for (int j = 0; j < W; ++j) v[j] = v0[DIRN * j];
-    return mr_recon<R>(v, sA, valid ? sel : 0);
+        for (int j = 0; j < W; ++j) v[j] = v0[DIRN * j];
+        const double w = mr_recon<R>(v, sA, valid ? sel : 0);
+        if (!small) value = w;
+    }
+    return value;
 }
 
 template <int R>

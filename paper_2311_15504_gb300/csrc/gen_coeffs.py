@@ -169,6 +169,18 @@ def generate() -> str:
         for row in bs:
             out.append("    " + ", ".join(hexlit(x) for x in row) + ",")
         out.append("};")
+        N = 2 * g - 2
+        out.append("// the same indicators as weights of the differences e_j (rows t, j = 0..2g-3),")
+        out.append("// and their orders m + n")
+        out.append(f"static __constant__ float kE{R}[{T * N}] = {{")
+        for m, n in lst:
+            k = m + n
+            row = [0] * N
+            for i in range(k):
+                row[g - 1 - m + i] = (-1) ** (k - 1 - i) * math.comb(k - 1, i)
+            out.append("    " + ", ".join(f"{x}.0f" for x in row) + ",")
+        out.append("};")
+        out.append(f"static __constant__ int kK{R}[{T}] = {{" + ", ".join(str(m + n) for m, n in lst) + "};")
         out.append(f"// a_l (same layout)")
         out.append(f"static __constant__ double kA{R}[{T * W}] = {{")
         for row in as_:
@@ -188,6 +200,8 @@ def generate() -> str:
         out.append(f"    __device__ static __forceinline__ double b(int i) {{ return kB{R}[i]; }}")
         out.append(f"    __device__ static __forceinline__ double a(int i) {{ return kA{R}[i]; }}")
         out.append(f"    __device__ static __forceinline__ const double *a_table() {{ return kA{R}; }}")
+        out.append(f"    __device__ static __forceinline__ const float *e() {{ return kE{R}; }}")
+        out.append(f"    __device__ static __forceinline__ int order(int t) {{ return kK{R}[t]; }}")
         for f in "WSD":
             out.append(f"    __device__ static __forceinline__ const float2 *{f.lower()}() {{ return k{f}{R}; }}")
         out.append("};")
