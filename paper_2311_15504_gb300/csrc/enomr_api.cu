@@ -426,16 +426,85 @@ __global__ void k_axpy(long long n, double a, const double *x, double *y, int ac
         y[i] = acc ? fma(a, x[i], y[i]) : a * x[i];
 }
 
-__global__ void k_set_dt(const double *smax, double cfl, double dt_fixed, double *dt)
+__device__ __forceinline__ double step_size(double sm, double cfl, double dt_fixed)
 {
     // a state without any wave speed (Burgers with u = 0) is steady: dt = 0;
     // a non-finite maximum (a non-physical state, flagged in the status
     // word) gives NaN, never a step that does not advance
-    const double sm = *smax;
-    *dt = dt_fixed > 0.0 ? dt_fixed
-                         : ((sm > 0.0 && sm < __longlong_as_double(0x7ff0000000000000LL))
-                                ? cfl / sm
-                                : (sm == 0.0 ? 0.0 : __longlong_as_double(0x7ff8000000000000LL)));
+    return dt_fixed > 0.0 ? dt_fixed
+                          : ((sm > 0.0 && sm < __longlong_as_double(0x7ff0000000000000LL))
+                                 ? cfl / sm
+                                 : (sm == 0.0 ? 0.0 : __longlong_as_double(0x7ff8000000000000LL)));
+}
+
+__global__ void k_set_dt(const double *smax, double cfl, double dt_fixed, double *dt)
+{
+    *dt = step_size(*smax, cfl, dt_fixed);
+}
+
+// 1D Euler: the three split speeds, the CFL speed and the step in one launch.
+// One cell per thread (a line this serves is short: the launch lasts as long
+// as one cell's speeds); a cell bitwise equal to its predecessor in the warp
+// repeats its speeds, and a warp of such cells evaluates none.
+__global__ void __launch_bounds__(128) k_line_speed(const double *U, long long n, double gm1,
+                                                    double gamma, double inv_dx, double cfl,
+                                                    double dt_fixed, double *alpha, double *smax,
+                                                    int *done, double *dt, int *status)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned long long w[4] = {0, 0, 0, 0};
+    const long long stride = (long long)gridDim.x * 128;
+    for (long long i0 = (long long)blockIdx.x * 128 + (threadIdx.x & ~31); i0 < n; i0 += stride) {
+        const long long i = i0 + lane;
+        const bool in = i < n;
+        double u[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) u[q] = in ? U[q * n + i] : 0.0;
+        bool same = lane > 0 || i0 > 0;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const double l = __shfl_up_sync(0xffffffffu, u[q], 1);
+            const double p = lane > 0 ? l : (i0 > 0 ? U[q * n + i - 1] : 0.0);
+            same = same && __double_as_longlong(p) == __double_as_longlong(u[q]);
+        }
+        if (in && !same) {
+            const CellWaves cw = cell_waves<3>(u[0], u[1], 0.0, u[2], gm1, gamma, status);
+            const double s[4] = {fabs(__dsub_rn(cw.u, cw.c)), fabs(cw.u), fabs(__dadd_rn(cw.u, cw.c)),
+                                 __dmul_rn(__dadd_rn(fabs(cw.u), cw.c), inv_dx)};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const unsigned long long b = (unsigned long long)__double_as_longlong(s[k]);
+                w[k] = w[k] > b ? w[k] : b;
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long x = __shfl_xor_sync(0xffffffffu, w[k], o);
+            w[k] = w[k] > x ? w[k] : x;
+        }
+        if (lane == k && w[k])
+            atomicMax((unsigned long long *)(k < 3 ? alpha + k : smax), w[k]);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(done, 1) == (int)gridDim.x - 1) {
+        __threadfence();
+        *dt = step_size(*(volatile double *)smax, cfl, dt_fixed);
+    }
+}
+
+cudaError_t launch_line_speed(const double *U, long long n, double gm1, double gamma,
+                              double inv_dx, double cfl, double dt_fixed, double *alpha,
+                              double *smax, int *done, double *dt, int *status, cudaStream_t s)
+{
+    long long blocks = (n + 127) / 128;
+    if (blocks > 152 * 16) blocks = 152 * 16;
+    k_line_speed<<<(unsigned)blocks, 128, 0, s>>>(U, n, gm1, gamma, inv_dx, cfl, dt_fixed, alpha,
+                                                  smax, done, dt, status);
+    return cudaGetLastError();
 }
 
 __global__ void k_advance_time(double *t, const double *dt, double mult)
@@ -943,8 +1012,10 @@ ENOMR_API enomr_status enomr_init(enomr_ctx **out, int eq, int ndim, int64_t nx,
     c->nstate = (long long)C * nx * ny;
     // one block: smax, counts (6 ints), ax, ay (up to here cleared by one
     // memset; in 1D without ay), then the tile lists and the block maps
-    const size_t zero_all = sizeof(double) * (4 + 3 * (size_t)ny + 3 * (size_t)nx);
-    c->zero_bytes = ndim == 2 ? zero_all : sizeof(double) * (4 + 3 * (size_t)ny);
+    // (in 1D ax holds the speeds of three stages)
+    const size_t nax = ndim == 2 ? 3 * (size_t)ny : 9;
+    const size_t zero_all = sizeof(double) * (4 + nax + 3 * (size_t)nx);
+    c->zero_bytes = ndim == 2 ? zero_all : sizeof(double) * (4 + nax);
     const long long nb = map_blocks(c);
     const long long lists = ((nx + X_TP - 2) / (X_TP - 1)) * ((ny + X_NL - 1) / X_NL) +
                             ((ny + Y_TP - 2) / (Y_TP - 1)) * ((nx + Y_NL - 1) / Y_NL) + nb;
@@ -974,7 +1045,7 @@ ENOMR_API enomr_status enomr_init(enomr_ctx **out, int eq, int ndim, int64_t nx,
     if (ok) {
         c->counts = (int *)(c->smax + 1);
         c->ax = c->smax + 4;
-        c->ay = c->ax + 3 * ny;
+        c->ay = c->ax + nax;
         if (mapped) {
             c->tile_lists = (int *)(c->ay + 3 * nx);
             c->flat = (unsigned char *)(c->tile_lists + lists);
@@ -1075,9 +1146,52 @@ static enomr_status set_step_dt(enomr_ctx *c, const double *U, double dt, double
     return cu(launch_set_dt(c->smax, cfl, 0.0, c->dt, c->stream));
 }
 
+// One SSP-RK3 step of 1D Euler in four launches: the speeds of U^n with the
+// step, and three stages of which the first two also take the speeds of the
+// state they make.  The last stage's speeds are left in c->ax.
+static enomr_status step_line(enomr_ctx *c, double *U, double dt, double cfl)
+{
+    if (!(dt > 0.0) && !(cfl > 0.0)) return ENOMR_EINVAL;
+    CU_TRY(cudaMemsetAsync(c->smax, 0, c->zero_bytes, c->stream));
+    double *alpha[3] = {c->ax + 3, c->ax + 6, c->ax};
+    prof_start(c, 3);
+    cudaError_t e = launch_line_speed(U, c->nx, c->gamma - 1.0, c->gamma, 1.0 / c->dx, cfl, dt,
+                                      alpha[0], c->smax, c->counts, c->dt, c->status, c->stream);
+    prof_stop(c, 3);
+    CU_TRY(e);
+    const double *from[3] = {U, c->U1, c->U2};
+    double *to[3] = {c->U1, c->U2, U};
+    for (int s = 0; s < 3; ++s) {
+        SweepArgs a = sweep_args(c, from[s], false);
+        a.alpha = alpha[s];
+        a.alpha_next = s < 2 ? alpha[s + 1] : nullptr;
+        a.epi.mode = EPI_STAGE;
+        a.epi.c0 = RK_C0[s];
+        a.epi.c1 = RK_C1[s];
+        a.epi.dt_dev = c->dt;
+        a.epi.Un = U;
+        a.epi.out = to[s];
+        prof_start(c, 1);
+        e = by_order<E1F>(c->order, a, c->stream);
+        prof_stop(c, 1);
+        CU_TRY(e);
+    }
+    return ENOMR_OK;
+}
+
 ENOMR_API enomr_status enomr_step(enomr_ctx *c, double *U, double dt, double cfl, double *dt_used)
 {
     if (!c || !U) return ENOMR_EINVAL;
+    if (c->eq == ENOMR_EULER && c->ndim == 1) {
+        enomr_status st = step_line(c, U, dt, cfl);
+        if (st) return st;
+        if (dt_used) {
+            CU_TRY(cudaMemcpyAsync(dt_used, c->dt, sizeof(double), cudaMemcpyDeviceToHost,
+                                   c->stream));
+            CU_TRY(cudaStreamSynchronize(c->stream));
+        }
+        return ENOMR_OK;
+    }
     enomr_status st = set_step_dt(c, U, dt, cfl, map_allowed(c) ? MAP_N : MAP_NONE);
     if (st) return st;
     // with a CFL step the alpha of U^n was just computed with the wave-speed max

@@ -219,6 +219,12 @@ template <int R> cudaError_t launch_advection_vjp(const AdvArgs &a, const double
 cudaError_t launch_alpha(int C, const AlphaArgs &a, cudaStream_t s);
 cudaError_t launch_scalar_speed(const double *U, long long n, double inv_dx, double *speed,
                                 double *smax, int *status, cudaStream_t s);
+// 1D Euler: max |u-c|, |u|, |u+c| into alpha[3] and the CFL speed into smax
+// (zeroed before, as is done), and the step: dt_fixed > 0, or cfl / smax, by
+// the last CTA
+cudaError_t launch_line_speed(const double *U, long long n, double gm1, double gamma,
+                              double inv_dx, double cfl, double dt_fixed, double *alpha,
+                              double *smax, int *done, double *dt, int *status, cudaStream_t s);
 cudaError_t launch_set_dt(const double *smax, double cfl, double dt_fixed, double *dt_dev,
                           cudaStream_t s);
 

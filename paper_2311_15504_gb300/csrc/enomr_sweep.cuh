@@ -117,6 +117,21 @@ __device__ __forceinline__ void side_cell(const SweepArgs &A, long long craw, lo
     if (kind == SIDE_REFLECTIVE) u[QN] = -u[QN];
 }
 
+// Back-projection of a 1D face (interface_flux, C = 3) from its field values
+// f^+ + f^-; every rounding is written out, so that each kernel of the 1D
+// equations has the same bits.
+__device__ __forceinline__ void back_project3(double uh, double Hh, double hq, double cs,
+                                              double b1, const double *ft, double *Fh)
+{
+    const double q = __dmul_rn(0.25, b1);
+    const double ph0 = __dmul_rn(q, ft[0]), pha = __dmul_rn(q, ft[2]);
+    const double ph1 = __dmul_rn(__dmul_rn(-0.5, b1), ft[1]);
+    const double s = __dadd_rn(ph0, pha), d = __dsub_rn(pha, ph0);
+    Fh[0] = __dadd_rn(s, ph1);
+    Fh[1] = __fma_rn(uh, Fh[0], __dmul_rn(cs, d));
+    Fh[2] = __fma_rn(Hh, s, __fma_rn(__dmul_rn(uh, cs), d, __dmul_rn(hq, ph1)));
+}
+
 // Flux of interface x_{k-1/2}, k = x0 + p, of tile line `line` into
 // t.Fh(., line, p) (and the selections / field values when requested).
 // FLATP: the interface is flat (both sides' centre triples of cell states
@@ -246,7 +261,14 @@ __device__ __forceinline__ void interface_flux(const SweepArgs &A, long long x0,
             q = fma(l0c, t.F(0, line, s), q);
         }
     };
+    double ft3[3] = {0.0, 0.0, 0.0};
     auto accumulate = [&](int f, double ft) {
+        if constexpr (C == 3) {
+            if (f == 0) ft3[0] = ft;
+            if (f == 1) ft3[1] = ft;
+            if (f == 2) ft3[2] = ft;
+            return;
+        }
         if (f == 0) {
             const double ph = 0.25 * b1 * ft;
             acc_s += ph;
@@ -358,10 +380,14 @@ __device__ __forceinline__ void interface_flux(const SweepArgs &A, long long x0,
         }
     }
     double Fh[C];
-    Fh[0] = acc_s + ph1;
-    Fh[1] = fma(uh, Fh[0], cs * acc_d);
-    if (C == 4) Fh[2] = fma(vh, Fh[0], ph2);
-    Fh[C - 1] = fma(Hh, acc_s, fma(uh * cs, acc_d, fma(hq, ph1, vh * ph2)));
+    if constexpr (C == 3) {
+        back_project3(uh, Hh, hq, cs, b1, ft3, Fh);
+    } else {
+        Fh[0] = acc_s + ph1;
+        Fh[1] = fma(uh, Fh[0], cs * acc_d);
+        Fh[2] = fma(vh, Fh[0], ph2);
+        Fh[C - 1] = fma(Hh, acc_s, fma(uh * cs, acc_d, fma(hq, ph1, vh * ph2)));
+    }
     // a lane without an interface of its own (it only votes) must not store
     // over the owner's slot; in the field-parallel form the first lane stores
     if (valid && fsel <= 0)
