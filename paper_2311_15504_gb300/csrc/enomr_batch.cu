@@ -55,17 +55,28 @@ __global__ void __launch_bounds__(128) k_batch_alpha(BatchAlphaArgs A)
         const long long n = A.n[tl.prob];
         const double *U = A.U + A.base[tl.prob];
         unsigned long long w[3] = {0, 0, 0};
+        // a cell bitwise equal to its predecessor has its speeds: only the
+        // others are evaluated, and a tile without any is done
+        bool any = false;
         for (int j = threadIdx.x; j < A.cells_per_tile; j += blockDim.x) {
             const long long i = (long long)tl.x0 + j;
             if (i < n) {
-                double s3[3];
-                wave_speeds3(U[i], U[n + i], U[2 * n + i], A.gm1, A.gamma, s3, A.status);
-                for (int k = 0; k < 3; ++k) {
-                    const unsigned long long b = __double_as_longlong(s3[k]);
-                    w[k] = w[k] > b ? w[k] : b;
+                const double u0 = U[i], u1 = U[n + i], u2 = U[2 * n + i];
+                const long long l = i > 0 ? i - 1 : 0;
+                if (i == 0 || __double_as_longlong(U[l]) != __double_as_longlong(u0) ||
+                    __double_as_longlong(U[n + l]) != __double_as_longlong(u1) ||
+                    __double_as_longlong(U[2 * n + l]) != __double_as_longlong(u2)) {
+                    double s3[3];
+                    wave_speeds3(u0, u1, u2, A.gm1, A.gamma, s3, A.status);
+                    any = true;
+                    for (int k = 0; k < 3; ++k) {
+                        const unsigned long long b = __double_as_longlong(s3[k]);
+                        w[k] = w[k] > b ? w[k] : b;
+                    }
                 }
             }
         }
+        if (!__syncthreads_or(any)) continue;
         for (int k = 0; k < 3; ++k) {
             for (int o = 16; o > 0; o >>= 1) {
                 const unsigned long long x = __shfl_xor_sync(0xffffffffu, w[k], o);

@@ -451,7 +451,8 @@ struct LongForm {
 template <int R, int C, int DIR, int TP, int NL, bool EXT = false,
           int LM = LongForm<DIR>::value, class Tile>
 __device__ __forceinline__ void sweep_tile(const SweepArgs &A, long long x0, long long l0,
-                                           const double *sA, const Tile &t)
+                                           const double *sA, const Tile &t,
+                                           unsigned long long *last = nullptr)
 {
     constexpr int g = (R + 1) / 2, S = TP + 2 * g - 1;
     constexpr int NT = TP * NL;
@@ -741,6 +742,8 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs &A, long long x0, lon
 
     // ---- flux difference and epilogue for the TP-1 cells of the tile
     unsigned long long ws[3] = {0, 0, 0};
+    double ov[3] = {0.0, 0.0, 0.0};  // C = 3: this cell's new state
+    bool new_state = false;
     if (p < TP - 1 && Lg < nlines) {
         const long long i = x0 + p;
         // cells of dead blocks are written by write_dead_block
@@ -787,15 +790,67 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs &A, long long x0, lon
             else
                 with_epilogue_form(A.epi, tile_form);
             if (C == 3 && A.alpha_next) {
-                double w3[3];
-                wave_speeds3(o[0], o[1], o[2], A.gm1, A.gamma, w3, A.status);
+                new_state = true;
 #pragma unroll
-                for (int k3 = 0; k3 < 3; ++k3) ws[k3] = __double_as_longlong(w3[k3]);
+                for (int q = 0; q < 3; ++q) ov[q] = o[q];
             }
         }
     }
     if (C == 3 && A.alpha_next) {
-        // CTA maximum of the new state's wave speeds -> the next stage's alpha
+        // CTA maximum of the new state's wave speeds -> the next stage's alpha.
+        // A cell bitwise equal to its predecessor in the tile has its speeds;
+        // the others are compacted (into the tile's flux and list storage) and
+        // evaluated by whole warps, about 45 FP64 operations each: a tile on
+        // one state takes one such warp instead of one per 32 cells.  A tile
+        // with a single state that this CTA evaluated last, for the same
+        // problem, adds nothing.
+        __syncthreads();  // the fluxes and the list are read no more
+        if (tid == 0) t.nrep() = 0;
+        if (new_state)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) t.Fh(q, 0, p) = ov[q];
+        __syncthreads();
+        bool first = new_state;
+        if (new_state && p > 0) {
+            bool same = true;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                same = same && __double_as_longlong(t.Fh(q, 0, p - 1)) == __double_as_longlong(ov[q]);
+            first = !same;
+        }
+        const unsigned need = __ballot_sync(FULL, first);
+        if (need) {
+            int base = 0;
+            if (lane == 0) base = atomicAdd(&t.nrep(), __popc(need));
+            base = __shfl_sync(FULL, base, 0);
+            if (first) t.list()[base + __popc(need & ((1u << lane) - 1u))] = p;
+        }
+        __syncthreads();
+        const int n = t.nrep();
+        bool known = false;
+        if (n == 1 && last && last[3] == (unsigned long long)A.alpha_next) {
+            known = true;
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+                known = known && last[q] == (unsigned long long)__double_as_longlong(t.Fh(q, 0, t.list()[0]));
+        }
+        __syncthreads();  // last is rewritten below
+        if (known) return;
+        if (last && n == 1 && tid == 0) {
+            for (int q = 0; q < 3; ++q) last[q] = (unsigned long long)__double_as_longlong(t.Fh(q, 0, t.list()[0]));
+            last[3] = (unsigned long long)A.alpha_next;
+        }
+        for (int b = tid & ~31; b < n; b += NT)
+            if (b + lane < n) {
+                const int i = t.list()[b + lane];
+                double w3[3];
+                wave_speeds3(t.Fh(0, 0, i), t.Fh(1, 0, i), t.Fh(2, 0, i), A.gm1, A.gamma, w3, A.status);
+#pragma unroll
+                for (int k3 = 0; k3 < 3; ++k3) {
+                    const unsigned long long w = (unsigned long long)__double_as_longlong(w3[k3]);
+                    ws[k3] = ws[k3] > w ? ws[k3] : w;
+                }
+            }
 #pragma unroll
         for (int k3 = 0; k3 < 3; ++k3) {
 #pragma unroll
@@ -926,6 +981,8 @@ __global__ void __launch_bounds__(TP) k_batch_stage(BatchArgs B)
     constexpr int g = (R + 1) / 2, W = 2 * g - 1, T = Tab<R>::T;
     __shared__ SweepSmem<R, 3, TP, 1> sm;
     __shared__ double sA[T * W];
+    __shared__ unsigned long long last[4];  // sweep_tile: last single state and its alpha_next
+    if (threadIdx.x == 0) last[3] = 0;
     load_a_table<R>(sA, threadIdx.x, TP);
     // work items of tiles_per_item consecutive tiles (each thread evaluates
     // that many interfaces per item), strided over the persistent grid
@@ -964,7 +1021,7 @@ __global__ void __launch_bounds__(TP) k_batch_stage(BatchArgs B)
         A.epi.Un = B.Un + base;
         A.epi.Dprev = nullptr;
         A.epi.out = B.out + base;
-        sweep_tile<R, 3, 0, TP, 1>(A, tl.x0, 0, sA, ClassicTile<R, 3, 0, TP, 1>{sm});
+        sweep_tile<R, 3, 0, TP, 1>(A, tl.x0, 0, sA, ClassicTile<R, 3, 0, TP, 1>{sm}, last);
     }
 }
 
