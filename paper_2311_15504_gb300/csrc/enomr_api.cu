@@ -426,17 +426,6 @@ __global__ void k_axpy(long long n, double a, const double *x, double *y, int ac
         y[i] = acc ? fma(a, x[i], y[i]) : a * x[i];
 }
 
-__device__ __forceinline__ double step_size(double sm, double cfl, double dt_fixed)
-{
-    // a state without any wave speed (Burgers with u = 0) is steady: dt = 0;
-    // a non-finite maximum (a non-physical state, flagged in the status
-    // word) gives NaN, never a step that does not advance
-    return dt_fixed > 0.0 ? dt_fixed
-                          : ((sm > 0.0 && sm < __longlong_as_double(0x7ff0000000000000LL))
-                                 ? cfl / sm
-                                 : (sm == 0.0 ? 0.0 : __longlong_as_double(0x7ff8000000000000LL)));
-}
-
 __global__ void k_set_dt(const double *smax, double cfl, double dt_fixed, double *dt)
 {
     *dt = step_size(*smax, cfl, dt_fixed);
@@ -594,6 +583,12 @@ template <int R> struct AdvF {
 };
 template <int R> struct BurgF {
     static cudaError_t run(const AdvArgs &a, cudaStream_t s) { return launch_burgers<R>(a, s); }
+};
+template <int R> struct SmallF {
+    static cudaError_t run(const SmallArgs &a, bool burgers, cudaStream_t s)
+    {
+        return launch_scalar_step<R>(a, burgers, s);
+    }
 };
 template <int R> struct E1F {
     static cudaError_t run(const SweepArgs &a, cudaStream_t s) { return launch_euler1d<R>(a, s); }
@@ -1179,11 +1174,42 @@ static enomr_status step_line(enomr_ctx *c, double *U, double dt, double cfl)
     return ENOMR_OK;
 }
 
+// One SSP-RK3 step of a short scalar line in one launch.
+static enomr_status step_small(enomr_ctx *c, double *U, double dt, double cfl)
+{
+    const bool burgers = c->eq == ENOMR_BURGERS;
+    if (!(dt > 0.0)) {
+        if (!(cfl > 0.0) || (!burgers && !(c->adv != 0.0))) return ENOMR_EINVAL;
+        dt = burgers ? 0.0 : cfl * c->dx / fabs(c->adv);
+    }
+    SmallArgs a;
+    a.U = U;
+    a.n = c->nx;
+    a.bc = c->bc;
+    a.a = burgers ? 1.0 : c->adv;
+    a.inv_h = 1.0 / c->dx;
+    a.cfl = cfl;
+    a.dt_fixed = dt;
+    for (int s = 0; s < 3; ++s) {
+        a.c0[s] = RK_C0[s];
+        a.c1[s] = RK_C1[s];
+    }
+    a.dt = c->dt;
+    a.speed = c->ax;
+    a.status = c->status;
+    prof_start(c, 1);
+    const cudaError_t e = by_order<SmallF>(c->order, a, burgers, c->stream);
+    prof_stop(c, 1);
+    return cu(e);
+}
+
 ENOMR_API enomr_status enomr_step(enomr_ctx *c, double *U, double dt, double cfl, double *dt_used)
 {
     if (!c || !U) return ENOMR_EINVAL;
-    if (c->eq == ENOMR_EULER && c->ndim == 1) {
-        enomr_status st = step_line(c, U, dt, cfl);
+    const bool line = c->eq == ENOMR_EULER && c->ndim == 1;
+    const bool small = c->eq != ENOMR_EULER && c->nx <= SMALL_CELLS;
+    if (line || small) {
+        enomr_status st = line ? step_line(c, U, dt, cfl) : step_small(c, U, dt, cfl);
         if (st) return st;
         if (dt_used) {
             CU_TRY(cudaMemcpyAsync(dt_used, c->dt, sizeof(double), cudaMemcpyDeviceToHost,

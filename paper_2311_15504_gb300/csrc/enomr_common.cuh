@@ -20,6 +20,18 @@ __device__ __forceinline__ bool below_1e300(double x)
     return (__double_as_longlong(x) & 0x7fffffffffffffffLL) < 0x7e37e43c8800759cLL;
 }
 
+// The step of a state whose CFL speed is sm.
+__device__ __forceinline__ double step_size(double sm, double cfl, double dt_fixed)
+{
+    // a state without any wave speed (Burgers with u = 0) is steady: dt = 0;
+    // a non-finite maximum (a non-physical state, flagged in the status
+    // word) gives NaN, never a step that does not advance
+    return dt_fixed > 0.0 ? dt_fixed
+                          : ((sm > 0.0 && sm < __longlong_as_double(0x7ff0000000000000LL))
+                                 ? cfl / sm
+                                 : (sm == 0.0 ? 0.0 : __longlong_as_double(0x7ff8000000000000LL)));
+}
+
 struct CellWaves {
     double u, v, c;  // normal and tangential velocity, sound speed
 };

@@ -110,6 +110,20 @@ struct AdvArgs {
     Epilogue epi;
 };
 
+// One SSP-RK3 step of a scalar line of at most SMALL_CELLS cells (enomr_scalar.cuh)
+constexpr int SMALL_CELLS = 1024, SMALL_THREADS = 512;
+struct SmallArgs {
+    double *U;             // [n], in place
+    long long n;
+    int bc;
+    double a, inv_h;       // advection speed; 1 / dx
+    double cfl, dt_fixed;  // dt_fixed > 0, or (Burgers) the CFL step
+    double c0[3], c1[3];
+    double *dt, *speed;    // the step used; Burgers: speed and signs of the last stage
+    int *status;
+};
+template <int R> cudaError_t launch_scalar_step(const SmallArgs &a, bool burgers, cudaStream_t s);
+
 struct AlphaArgs {
     const double *U;
     long long nx, ny;

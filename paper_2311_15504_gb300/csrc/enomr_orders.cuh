@@ -71,6 +71,7 @@ template <int R> cudaError_t launch_euler2d_y(const SweepArgs &a, bool low, cuda
 
 template cudaError_t launch_advection<ENOMR_R>(const AdvArgs &, cudaStream_t);
 template cudaError_t launch_burgers<ENOMR_R>(const AdvArgs &, cudaStream_t);
+template cudaError_t launch_scalar_step<ENOMR_R>(const SmallArgs &, bool, cudaStream_t);
 template cudaError_t launch_euler1d<ENOMR_R>(const SweepArgs &, cudaStream_t);
 // with boundary sides / body force (the 2D problems of Sec. 4.4)
 template <int R> cudaError_t launch_euler2d_x_ext(const SweepArgs &a, bool low, cudaStream_t s)

@@ -62,3 +62,27 @@ def test_scalar_float_form(eq, order, n):
         flux = 0.5 * np.abs(u).max() ** 2 * (2 if burgers else 0) + np.abs(u).max()
         assert close(a, b, flux / h, order), (name, eq)
         s.check_status()
+
+
+@pytest.mark.parametrize("n", (18, 31, 32, 33, 200, 511, 512, 513, 1023, 1024, 1025))
+@pytest.mark.parametrize("order", (5, 17))
+@pytest.mark.parametrize("eq", ("advection", "advection_left", "burgers", "burgers_left",
+                                "burgers_mixed"))
+def test_short_line_step_equals_its_stages(eq, order, n):
+    """enomr_step of at most 1024 cells is one launch; its stages are one each."""
+    from paper_2311_15504_gb300 import enomr
+    h = 2.0 / n
+    u = lines(n)["plateau"]
+    u = -u if eq == "burgers_left" else (u - 1.0 if eq == "burgers_mixed" else u)
+    for bc in (enomr.PERIODIC, enomr.TRANSMISSIVE):
+        s = enomr.Solver(enomr.BURGERS if eq.startswith("burgers") else enomr.ADVECTION, n,
+                         order=order, dx=h, bc=bc, adv_speed=-0.7 if eq.endswith("left") else 1.0)
+        U = torch.from_numpy(u).cuda()
+        a, b, v = torch.empty_like(U), torch.empty_like(U), U.clone()
+        dt = s.cfl_dt(U, 0.4)
+        s.stage(1, U, U, a, dt)
+        s.stage(2, U, a, b, dt)
+        s.stage(3, U, b, a, dt)
+        assert s.step(v, 0.0, 0.4, return_dt=True) == dt
+        assert torch.equal(a, v)
+        s.check_status()
