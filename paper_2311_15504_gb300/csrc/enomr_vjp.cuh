@@ -53,6 +53,7 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
     __shared__ double sRow[NL][TP][3];
     __shared__ double sRowA[NL][TP][4];
     __shared__ double sRoeB[NL][TP][2][C];
+    __shared__ double sG[NL][TP][2 * C];
     __shared__ double sA[T * W];
 
     const long long nx = A.nx, ny = A.ny, ncell = nx * ny;
@@ -155,6 +156,25 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
     const double ph2_b = (C == 4) ? Fb[2] + FbE * vh : 0.0;
     const double ph0_b = acc_s_b - acc_d_b, pha_b = acc_s_b + acc_d_b;
 
+    // Component sums of the window with the weights of the full stencil on both
+    // sides.  A field with that choice (nearly all in smooth flow) has its sums
+    // over the window, and its part of the cells' cotangents, in common with the
+    // others up to factors of the field: X and Y once instead of eight sums per
+    // field, and one gather of G (below) instead of one per field.  What the
+    // windows on other choices differ by goes through the per-field path.  (FP64
+    // pipe bound: about half the operations.  Vortex with weak waves, 512^2,
+    // order 9, rollout of two steps and its gradient: 16.1 -> 13.1 ms.)
+    double X[C], Y[C], GU[C], GF[C];
+#pragma unroll
+    for (int q = 0; q < C; ++q) {
+        X[q] = Y[q] = GU[q] = GF[q] = 0.0;
+#pragma unroll
+        for (int j = 0; j < 2 * g; ++j) {
+            X[q] = fma(Coef<R>::m()[j], sU[q][line][p + j], X[q]);
+            Y[q] = fma(Coef<R>::p()[j], sF[q][line][p + j], Y[q]);
+        }
+    }
+
     double ftv[C];
     double hq_b = 0.0, uh_b = 0.0, vh_b = 0.0, kap_b = 0.0, c2g_b = 0.0;
     double ab[3] = {0.0, 0.0, 0.0};
@@ -232,41 +252,73 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
         else if (f == C - 1) ftb = 0.25 * b1 * pha_b;
         else if (shear) ftb = 0.5 * ph2_b;
         else ftb = -0.5 * b1 * ph1_b;
-        // effective reconstruction weights of the frozen choice, times ftb
-        constexpr int c0 = g - 1;
-        double wp[W], wm[W];
-#pragma unroll
-        for (int j = 0; j < W; ++j) {
-            wp[j] = (selp < T) ? sA[selp * W + j] * ftb : 0.0;
-            wm[j] = (selm < T) ? sA[selm * W + j] * ftb : 0.0;
+        // reverse of split and projection, per window cell.  With P, M the
+        // weights of the two sides times ftb and d = P - M, the cotangents are
+        // w_bar = alpha d and q_bar = P + M; the sums S[q] = sum_j d_j U_j[q]
+        // give both the U part of the row-coefficient cotangents (alpha S) and
+        // the alpha cotangent sum_j d_j w_j = l . S.
+        double S0 = ftb * X[0], S1 = ftb * X[1], ST = C == 4 ? ftb * X[2 % C] : 0.0,
+               SE = ftb * X[C - 1];
+        double Q0 = ftb * Y[0], Q1 = ftb * Y[1], QT = C == 4 ? ftb * Y[2 % C] : 0.0;
+        {
+            const double fa = ftb * alpha;
+            GU[0] = fma(fa, l0c, GU[0]);
+            GF[0] = fma(ftb, l0c, GF[0]);
+            if (shear) {
+                GU[2 % C] += fa;
+                GF[2 % C] += ftb;
+            } else {
+                GU[1] = fma(fa, l1c, GU[1]);
+                GF[1] = fma(ftb, l1c, GF[1]);
+                GU[C - 1] += fa;
+                GF[C - 1] += ftb;
+                if (C == 4) {
+                    GU[2 % C] = fma(-vh, fa, GU[2 % C]);
+                    GF[2 % C] = fma(-vh, ftb, GF[2 % C]);
+                }
+            }
         }
-        if (selp == T) { wp[c0] = 0.5 * ftb; wp[c0 + 1] = 0.5 * ftb; }
-        if (selp == T + 1) { wp[c0] = 1.5 * ftb; wp[c0 - 1] = -0.5 * ftb; }
-        if (selp == T + 2) wp[c0] = ftb;
-        if (selm == T) { wm[c0] = 0.5 * ftb; wm[c0 + 1] = 0.5 * ftb; }
-        if (selm == T + 1) { wm[c0] = 1.5 * ftb; wm[c0 - 1] = -0.5 * ftb; }
-        if (selm == T + 2) wm[c0] = ftb;
-        // reverse of split and projection, per window cell.  With d = P - M
-        // the cotangents are w_bar = alpha d and q_bar = P + M; the sums
-        // S[q] = sum_j d_j U_j[q] give both the U part of the row-coefficient
-        // cotangents (alpha S) and the alpha cotangent sum_j d_j w_j = l . S.
-        double S0 = 0.0, S1 = 0.0, ST = 0.0, SE = 0.0, Q0 = 0.0, Q1 = 0.0, QT = 0.0;
+        const bool other = owned && (selp | selm) != 0;
+        const bool others = __syncthreads_or(other) != 0;
+        if (others) {
+            // the frozen choice's weights minus the full stencil's, times ftb
+            constexpr int c0 = g - 1;
+            double wp[W], wm[W];
 #pragma unroll
-        for (int j = 0; j < 2 * g; ++j) {
-            const int s = p + j;
-            const double P = (j <= 2 * g - 2) ? wp[j] : 0.0;
-            const double M = (j >= 1) ? wm[2 * g - 1 - j] : 0.0;
-            const double qb = P + M, d = P - M;
-            sWB[line][p][j] = d;  // alpha is folded into the gather's row
-            sQB[line][p][j] = qb;
-            S0 = fma(d, sU[0][line][s], S0);
-            Q0 = fma(qb, sF[0][line][s], Q0);
-            if (C == 4) ST = fma(d, sU[2][line][s], ST);
-            if (!shear) {
-                S1 = fma(d, sU[1][line][s], S1);
-                SE = fma(d, sU[C - 1][line][s], SE);
-                Q1 = fma(qb, sF[1][line][s], Q1);
-                if (C == 4) QT = fma(qb, sF[2][line][s], QT);
+            for (int j = 0; j < W; ++j) {
+                double a = (selp < T) ? sA[selp * W + j] : 0.0, b = (selm < T) ? sA[selm * W + j] : 0.0;
+                if (j == c0) {
+                    a = selp == T ? 0.5 : (selp == T + 1 ? 1.5 : (selp == T + 2 ? 1.0 : a));
+                    b = selm == T ? 0.5 : (selm == T + 1 ? 1.5 : (selm == T + 2 ? 1.0 : b));
+                }
+                if (j == c0 + 1) {
+                    a = selp == T ? 0.5 : a;
+                    b = selm == T ? 0.5 : b;
+                }
+                if (j == c0 - 1) {
+                    a = selp == T + 1 ? -0.5 : a;
+                    b = selm == T + 1 ? -0.5 : b;
+                }
+                wp[j] = other ? (a - sA[j]) * ftb : 0.0;
+                wm[j] = other ? (b - sA[j]) * ftb : 0.0;
+            }
+#pragma unroll
+            for (int j = 0; j < 2 * g; ++j) {
+                const int s = p + j;
+                const double P = (j <= 2 * g - 2) ? wp[j] : 0.0;
+                const double M = (j >= 1) ? wm[2 * g - 1 - j] : 0.0;
+                const double qb = P + M, d = P - M;
+                sWB[line][p][j] = d;  // alpha is folded into the gather's row
+                sQB[line][p][j] = qb;
+                S0 = fma(d, sU[0][line][s], S0);
+                Q0 = fma(qb, sF[0][line][s], Q0);
+                if (C == 4) ST = fma(d, sU[2][line][s], ST);
+                if (!shear) {
+                    S1 = fma(d, sU[1][line][s], S1);
+                    SE = fma(d, sU[C - 1][line][s], SE);
+                    Q1 = fma(qb, sF[1][line][s], Q1);
+                    if (C == 4) QT = fma(qb, sF[2][line][s], QT);
+                }
             }
         }
         double l0b, l1b = 0.0, ltb = 0.0;
@@ -282,6 +334,7 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
             ab[aidx] += a;
         }
         // gather rows: U part scaled by alpha (it multiplies d), F part not
+        if (others) {
         sRow[line][p][0] = l0c;
         sRow[line][p][1] = l1c;
         sRow[line][p][2] = (C == 4) ? -vh : 0.0;
@@ -289,6 +342,7 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
         sRowA[line][p][1] = alpha * l1c;
         sRowA[line][p][2] = (C == 4) ? -alpha * vh : 0.0;
         sRowA[line][p][3] = alpha;
+        }
         // row coefficients -> Roe scalars
         if (shear) {
             vh_b -= l0b;
@@ -308,6 +362,7 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
             uh_b -= l1b;
             vh_b -= ltb;
         }
+        if (!others) continue;
         __syncthreads();
         // gather: staged cell s receives wb l and qb l from interfaces p' = s - j
 #pragma unroll
@@ -351,6 +406,39 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
             }
         }
         __syncthreads();
+    }
+
+    // ---- the common part of the fields: cell s receives the full stencil's
+    // weight of its place in the window of interface p' = s - j times G
+#pragma unroll
+    for (int q = 0; q < C; ++q) {
+        sG[line][p][q] = GU[q];
+        sG[line][p][C + q] = GF[q];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < CPT; ++c) {
+        const int idx = tid + c * NT;
+        if (idx < NL * S) {
+            int gl, s;
+            if (DIR == 0) {
+                gl = idx / S;
+                s = idx - gl * S;
+            } else {
+                s = idx / NL;
+                gl = idx - s * NL;
+            }
+#pragma unroll
+            for (int j = 0; j < 2 * g; ++j) {
+                const int pp = s - j;
+                if (pp < 0 || pp >= TP) continue;
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    cUb[c][q] = fma(Coef<R>::m()[j], sG[gl][pp][q], cUb[c][q]);
+                    cFb[c][q] = fma(Coef<R>::p()[j], sG[gl][pp][C + q], cFb[c][q]);
+                }
+            }
+        }
     }
 
     // ---- reverse of the back-projection terms that need the field values

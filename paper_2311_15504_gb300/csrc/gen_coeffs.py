@@ -13,18 +13,11 @@ and the indicator of Eq. (CurrentIS), h^K P^(K) with K = m+n, is the
 
     b_s = sum_{i > s} (K+1)! / prod_{k != i} (xi_i - xi_k).
 
-Two further forms of the interface-value weights multiply the differences
+A second form of the interface-value weights multiplies the differences
 e_j = f_{j+1} - f_j of neighbouring cells instead of the cells.  As the a_l of a
 stencil add up to 1, sum_l a_l f_{c+l} = f_c + sum_j w_j e_j with
 
-    w_j = sum_{l > j} a_l  (j >= c),    w_j = -sum_{l <= j} a_l  (j < c),
-
-and with the full stencil on both sides of an interface (window a_l and its
-mirror image over 2g cells, middle pair g-1, g) the sum and the difference of
-the two reconstructions are
-
-    1/2 sum (a_j + a_{2g-1-j}) f_j = 1/2 (f_{g-1} + f_g) + sum_j s_j e_j,
-        sum (a_j - a_{2g-1-j}) f_j = sum_j d_j e_j.
+    w_j = sum_{l > j} a_l  (j >= c),    w_j = -sum_{l <= j} a_l  (j < c).
 
 They are written as pairs of floats, high part (rounded to nearest) and rest.
 
@@ -99,15 +92,6 @@ def difference_weights(rowa, c: int):
     W = len(rowa)
     return [(sum(rowa[j + 1:], Fraction(0)) if j >= c else -sum(rowa[:j + 1], Fraction(0)))
             for j in range(W - 1)]
-
-
-def face_weights(rowa):
-    """s_j and d_j, j = 0 .. 2g-2, of the full window row."""
-    a = list(rowa) + [Fraction(0)]
-    n, g = len(a), len(a) // 2
-    t = [(a[j] + a[n - 1 - j]) / 2 - (Fraction(1, 2) if j in (g - 1, g) else 0) for j in range(n)]
-    d = [a[j] - a[n - 1 - j] for j in range(n)]
-    return [[-sum(v[:j + 1], Fraction(0)) for j in range(n - 1)] for v in (t, d)]
 
 
 def to_float(x: Fraction) -> Fraction:
@@ -186,9 +170,13 @@ def generate() -> str:
         for row in as_:
             out.append("    " + ", ".join(hexlit(x) for x in row) + ",")
         out.append("};")
-        out.append("// {high, rest} of the difference weights w_j of every row, of s_j and of d_j")
-        for name, rows in ((f"kW{R}", [difference_weights(r, g - 1) for r in as_]),
-                           (f"kS{R}", face_weights(as_[0])[:1]), (f"kD{R}", face_weights(as_[0])[1:])):
+        full = list(as_[0]) + [Fraction(0)]
+        out.append("// full stencil: a_j + a_{2g-1-j} and a_j - a_{2g-1-j}, j = 0..2g-1")
+        for name, sg in ((f"kP{R}", 1), (f"kM{R}", -1)):
+            out.append(f"static __constant__ double {name}[{2 * g}] = {{"
+                       + ", ".join(hexlit(full[j] + sg * full[2 * g - 1 - j]) for j in range(2 * g)) + "};")
+        out.append("// {high, rest} of the difference weights w_j of every row")
+        for name, rows in ((f"kW{R}", [difference_weights(r, g - 1) for r in as_]),):
             out.append(f"static __constant__ float2 {name}[{sum(len(r) for r in rows)}] = {{")
             for row in rows:
                 out.append("    " + ", ".join("{%s, %s}" % tuple(map(flit, pair(x))) for x in row) + ",")
@@ -202,7 +190,9 @@ def generate() -> str:
         out.append(f"    __device__ static __forceinline__ const double *a_table() {{ return kA{R}; }}")
         out.append(f"    __device__ static __forceinline__ const float *e() {{ return kE{R}; }}")
         out.append(f"    __device__ static __forceinline__ int order(int t) {{ return kK{R}[t]; }}")
-        for f in "WSD":
+        for f in "PM":
+            out.append(f"    __device__ static __forceinline__ const double *{f.lower()}() {{ return k{f}{R}; }}")
+        for f in "W":
             out.append(f"    __device__ static __forceinline__ const float2 *{f.lower()}() {{ return k{f}{R}; }}")
         out.append("};")
     out.append("")
