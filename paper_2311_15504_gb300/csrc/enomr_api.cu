@@ -508,21 +508,43 @@ __global__ void __launch_bounds__(256) k_scalar_speed(const double *U, long long
                                                       double *speed, double *smax, int *status)
 {
     unsigned long long m = 0, fl = 0;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const long long b = __double_as_longlong(U[i]);
+    auto take = [&](double u) {
+        const long long b = __double_as_longlong(u);
         const unsigned long long a = (unsigned long long)(b & 0x7fffffffffffffffLL);
-        if (!below_1e300(U[i])) atomicOr(status, ST_NONPHYS_CELL);
+        if (!below_1e300(u)) atomicOr(status, ST_NONPHYS_CELL);
         m = m > a ? m : a;
         if (a != 0) fl |= (b < 0) ? SGN_NEG : SGN_POS;
+    };
+    // eight loads in flight per thread: the launch is bound by the latency of
+    // its reads otherwise (N = 2^22: 21 us with one)
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    for (; i + 7 * stride < n; i += 8 * stride) {
+        double u[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) u[j] = U[i + j * stride];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) take(u[j]);
     }
+    for (; i < n; i += stride) take(U[i]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long w = __shfl_xor_sync(0xffffffffu, m, o);
         m = m > w ? m : w;
         fl |= __shfl_xor_sync(0xffffffffu, fl, o);
     }
+    // one CTA, one atomic each: the launch's warps would queue on the address
+    __shared__ unsigned long long sm[8], sf[8];
     if ((threadIdx.x & 31) == 0) {
+        sm[threadIdx.x >> 5] = m;
+        sf[threadIdx.x >> 5] = fl;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) {
+            m = m > sm[w] ? m : sm[w];
+            fl |= sf[w];
+        }
         atomicMax((unsigned long long *)speed, m);
         if (fl) atomicOr((unsigned long long *)(speed + 1), fl);
         if (smax) {
@@ -535,7 +557,8 @@ __global__ void __launch_bounds__(256) k_scalar_speed(const double *U, long long
 cudaError_t launch_scalar_speed(const double *U, long long n, double inv_dx, double *speed,
                                 double *smax, int *status, cudaStream_t s)
 {
-    long long blocks = (n + 255) / 256;
+    long long blocks = (n + 2047) / 2048;  // eight cells per thread
+    if (blocks < 1) blocks = 1;
     if (blocks > 152 * 8) blocks = 152 * 8;
     k_scalar_speed<<<(unsigned)blocks, 256, 0, s>>>(U, n, inv_dx, speed, smax, status);
     return cudaGetLastError();

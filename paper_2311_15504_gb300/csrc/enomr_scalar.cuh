@@ -83,12 +83,20 @@ __device__ __forceinline__ void load_w_table(float2 *sW, int tid, int nthreads)
     for (int i = tid; i < Tab<R>::T * N; i += nthreads) sW[i] = Coef<R>::w()[i];
 }
 
+// Resident CTAs (of 256 threads) per SM of the scalar kernels, 32 registers:
+// between the FP64 operations lie long float sums, and more warps fill the
+// FP64 pipe's gaps although the sums spill.  Burgers, N = 2^22, order 9 / 13 /
+// 17: 123 / 167 / 277 us a launch unbounded (58 to 84 registers), 117 / 141 /
+// 196 with five, 114 / 127 / 181 with eight; advection, N = 1 048 573, order 17:
+// 65 -> 52.
+constexpr int SCALAR_CTAS = 8;
+
 // ---------------------------------------------------------------------------
 // Scalar advection f(u) = a u, alpha = |a|: f^+ = a u, f^- = 0 for a >= 0
 // (mirror for a < 0).  One thread per interface.
 // ---------------------------------------------------------------------------
 template <int R, int TP>
-__global__ void __launch_bounds__(TP) k_advection(AdvArgs A)
+__global__ void __launch_bounds__(TP, SCALAR_CTAS) k_advection(AdvArgs A)
 {
     constexpr int g = (R + 1) / 2, W = 2 * g - 1, S = TP + 2 * g - 1, T = Tab<R>::T;
     __shared__ double sf[S];
@@ -137,7 +145,7 @@ __global__ void __launch_bounds__(TP) k_advection(AdvArgs A)
 // interface; split values are formed as written, 1/2 (f +- alpha u).
 // ---------------------------------------------------------------------------
 template <int R, int TP>
-__global__ void __launch_bounds__(TP) k_burgers(AdvArgs A)
+__global__ void __launch_bounds__(TP, SCALAR_CTAS) k_burgers(AdvArgs A)
 {
     constexpr int g = (R + 1) / 2, W = 2 * g - 1, S = TP + 2 * g - 1, T = Tab<R>::T;
     __shared__ double sp[S];
