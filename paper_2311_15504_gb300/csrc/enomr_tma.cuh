@@ -64,6 +64,7 @@ template <int R, int C, int DIR, int TP, int NL, bool SP = false>
 struct TmaTile {
     using SM = TmaSmem<R, C, DIR, TP, NL, SP>;
     static constexpr bool kLoads = false;
+    static constexpr bool kFloatSelect = true;
     // SP false: sqrt(rho), u_n, u_t, H are evaluated where an interface needs
     // them (the two centre cells of an interface that is not flat on one
     // state), not staged: 9 KB less shared memory per tile and no staging
