@@ -58,6 +58,9 @@ struct TileMap {
     unsigned char *dead;        // [nby][nbx]
     int nbx, nby;
     long long nx, ny;
+    double *dt;                 // optional: the CFL step, cfl / *smax, is stored here
+    const double *smax;
+    double cfl;
     int closed;                 // blocks at the edges of the domain are never dead
     int *tiles_x, *tiles_y, *blocks;
     int *count;                 // [3], zeroed before the launch: x tiles, y tiles, dead blocks
