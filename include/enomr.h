@@ -239,10 +239,13 @@ ENOMR_API enomr_status enomr_get_status(enomr_ctx *ctx);
 /*
  * enomr_set_staging -- how the 2D Euler sweeps bring a tile of cells (with
  * its g-cell halos, Sec. 2.1) into shared memory:
- *   ENOMR_STAGING_AUTO  (default) both sweeps by TMA where the state
- *                       allows it (nx even, U 16-byte aligned, no boundary
- *                       sides or body force; the faster staging for both
- *                       sweeps on GB300), otherwise plain loads;
+ *   ENOMR_STAGING_AUTO  (default) plain loads where the sweeps go by a list
+ *                       of tiles (grids of at least 2^16 cells without
+ *                       boundary sides or a body force: their tiles' costs
+ *                       differ, and one CTA per tile balances them better),
+ *                       else TMA where the state allows it (nx even, U
+ *                       16-byte aligned, no sides or body force), otherwise
+ *                       plain loads;
  *   ENOMR_STAGING_LOADS plain coalesced loads by the CTA's threads;
  *   ENOMR_STAGING_TMA   the TMA path only: calls whose state does not allow
  *                       it return ENOMR_EINVAL.
@@ -263,12 +266,13 @@ ENOMR_API enomr_status enomr_set_staging(enomr_ctx *ctx, int mode);
  *                         long path's windows stay in registers): for grids
  *                         of few tiles, whose launches last as long as a
  *                         few tiles in sequence;
- *   ENOMR_OCCUPANCY_AUTO  (default) LOW when the x sweep has fewer tiles
- *                         than four waves of the HIGH instance (grids up to
- *                         about 900^2), else HIGH.
- * On smooth data, where every interface takes the long path, LOW with TMA
- * staging is the fastest instance (about 4 % on a 4096^2 vortex); on
- * piecewise-constant data HIGH is (LOW is 40 % slower there).
+ *   ENOMR_OCCUPANCY_AUTO  (default) HIGH where the sweeps go by a list of
+ *                         tiles (enomr_set_staging); over all tiles LOW when
+ *                         the x sweep has fewer of them than four waves of
+ *                         the HIGH instance (grids up to about 900^2), else
+ *                         HIGH.
+ * On smooth data the two are alike (1024^2 vortex: 6.67 / 6.73 ms a step); on
+ * piecewise-constant data HIGH is faster (4096^2, order 9: 2.95 / 4.08 ms).
  * Same results bit for bit.  Host-only setting, no synchronisation.
  */
 enum { ENOMR_OCCUPANCY_AUTO = 0, ENOMR_OCCUPANCY_HIGH = 1, ENOMR_OCCUPANCY_LOW = 2 };
