@@ -211,6 +211,43 @@ def sweep_work(order, C, sel, n_interfaces, counts, stage_epilogue=False):
     return float(w[1]), float(w[0])
 
 
+def dead_cells(U):
+    """Cells of a 2D state in 32 x 32 blocks that hold one state together with
+    the eight blocks around them: the column sweep evaluates their stage
+    combination once per warp, not per cell."""
+    import torch
+    d = torch.zeros(U.shape[1:], dtype=torch.bool, device=U.device)
+    d[:, 1:] |= (U[:, :, 1:] != U[:, :, :-1]).any(dim=0)
+    d[1:] |= (U[:, 1:] != U[:, :-1]).any(dim=0)
+    live = torch.nn.functional.max_pool2d(d[None, None].float(), 32, ceil_mode=True)
+    live = torch.nn.functional.max_pool2d(live, 3, stride=1, padding=1)[0, 0] > 0
+    cells = live.repeat_interleave(32, 0).repeat_interleave(32, 1)[:U.shape[1], :U.shape[2]]
+    return int((~cells).sum().item())
+
+
+def executed_work(order, C, sel, n_interfaces, counts, n_dead=0, stage_epilogue=False):
+    """(flops, FP64 operations) that a sweep executes: sweep_work without the
+    indicators, which the sweeps form in float from 2g - 2 FP64 differences per
+    window (the windows that the float bound leaves open are not counted), and
+    without the stage combination of dead cells."""
+    import oracle  # table sizes only
+    fl, ops = sweep_work(order, C, sel, n_interfaces, counts, stage_epilogue)
+    g, T = (order + 1) // 2, oracle.num_tested(order)
+    sizes = np.array([oracle.candidate(order, t)[0] + oracle.candidate(order, t)[1] + 1
+                      for t in range(T)], dtype=np.float64)
+    cnt = np.asarray(sel, dtype=np.float64).copy()
+    cnt[T + 2] -= 2 * C * counts[0]
+    walk, walk_fl = np.cumsum(sizes), np.cumsum(2 * sizes - 1)
+    full = cnt[T] + cnt[T + 1]
+    windows = float(cnt.sum())
+    ops -= float(cnt[:T] @ walk + full * walk[-1]) + windows * (6 - (2 * g - 2))
+    fl -= float(cnt[:T] @ walk_fl + full * walk_fl[-1]) + windows * (8 - (2 * g - 2))
+    if stage_epilogue:
+        ops -= n_dead * 7 * C / 3
+        fl -= n_dead * 4 * C
+    return fl, ops
+
+
 # Tile shapes of the 2D sweeps (cells along the line, lines): row sweep,
 # column sweep.  Each tile writes TP - 1 cells of each of its lines and stages
 # g cells beyond them on either side.
@@ -476,9 +513,10 @@ def sweep_fracs(enomr, solver, U, order, n, cfl, peak_ops, steps=2, probe_ops=No
     hx = torch.bincount(sel[:nsx].long(), minlength=T + 3).cpu().numpy()
     hy = torch.bincount(sel[nsx:].long(), minlength=T + 3).cpu().numpy()
     nint = n * (n + 1)
-    work = {"x": (sweep_work(order, 4, hx, nint, sweep_counts(U, 0, order)),
+    work = {"x": (executed_work(order, 4, hx, nint, sweep_counts(U, 0, order)),
                   sweep_work(order, 4, hx, nint, (0, 0, 0, n * n))),
-            "y": (sweep_work(order, 4, hy, nint, sweep_counts(U, 1, order), stage_epilogue=True),
+            "y": (executed_work(order, 4, hy, nint, sweep_counts(U, 1, order), dead_cells(U),
+                                stage_epilogue=True),
                   sweep_work(order, 4, hy, nint, (0, 0, 0, n * n), stage_epilogue=True))}
     out = {}
     for kind, key in ((1, "x"), (2, "y")):
@@ -502,25 +540,19 @@ def sweep_fracs(enomr, solver, U, order, n, cfl, peak_ops, steps=2, probe_ops=No
 
 def scalar_work(order, sel, n, staged_ops):
     """Executed FP64 operations of one scalar (advection or Burgers) launch
-    on n cells: per interface the staged split value (staged_ops), the
-    baseline indicator (6), the indicators of the tested candidates up to
-    the chosen one (|S| each), the reconstruction (2g-1 for a tested
-    stencil, 1 for minmod), the flux difference (2) and the stage update
+    on n cells: per interface the staged split value (staged_ops), its
+    difference from the next (1), the value (2 for a tested stencil, whose sum
+    runs on float pairs in smooth flow; 1 for minmod; the indicators are
+    formed in float), the flux difference (2) and the stage update
     (7/3: the mean of the three SSP-RK3 stages, U + dt D in the first with
     1 fma, 2 fma and 1 mul in the others); only the window that carries the
     flux (f^+ for a > 0, u > 0) is evaluated.  sel: histogram of that
     side's selections."""
     import oracle  # table sizes only
-    g = (order + 1) // 2
     T = oracle.num_tested(order)
-    sizes = np.array([oracle.candidate(order, t)[0] + oracle.candidate(order, t)[1] + 1
-                      for t in range(T)], dtype=np.float64)
-    cum = np.cumsum(sizes)
     cnt = np.asarray(sel, dtype=np.float64)
-    w = float(n + 1) * (staged_ops + 6) + float(n) * (2 + 7 / 3)
-    for t in range(T):
-        w += cnt[t] * (cum[t] + (2 * g - 1))
-    w += (cnt[T] + cnt[T + 1]) * (cum[-1] + 1) + cnt[T + 2] * 1
+    w = float(n + 1) * (staged_ops + 1) + float(n) * (2 + 7 / 3)
+    w += 2 * cnt[:T].sum() + cnt[T:].sum()
     return w
 
 
@@ -964,6 +996,7 @@ def main_ours(a):
         hy = np.zeros(T + 3)
         cx = np.zeros(5)
         cy = np.zeros(5)
+        n_dead = 0
         ns = 0
         for it in range(a.steps):
             if it % every == 0:
@@ -972,13 +1005,14 @@ def main_ours(a):
                 hy += torch.bincount(sel[nsx:].long(), minlength=T + 3).cpu().numpy()
                 cx += np.array(sweep_counts(Us, 0, R))
                 cy += np.array(sweep_counts(Us, 1, R))
+                n_dead += dead_cells(Us)
                 ns += 1
             s.step(Us, 0.0, a.cfl)
         hx, hy, cx, cy = hx / ns, hy / ns, cx / ns, cy / ns
         del Us
         nint = n * (n + 1)
-        wx = sweep_work(R, 4, hx, nint, cx)
-        wy = sweep_work(R, 4, hy, nint, cy, stage_epilogue=True)
+        wx = executed_work(R, 4, hx, nint, cx)
+        wy = executed_work(R, 4, hy, nint, cy, n_dead / ns, stage_epilogue=True)
         mx = sweep_work(R, 4, hx, nint, (0, 0, 0, n * n))
         my = sweep_work(R, 4, hy, nint, (0, 0, 0, n * n), stage_epilogue=True)
         extras["flat_interface_fraction"] = [cx[0] / nint, cy[0] / nint]
