@@ -165,9 +165,10 @@ static enomr_status batch_alpha_dt(enomr_batch *b, const double *U, double cfl, 
     a.base = b->base;
     a.n = b->n;
     a.inv_dx = b->inv_dx;
-    a.tiles = b->tiles[b->tp_index];
-    a.ntiles = b->ntiles[b->tp_index];
-    a.cells_per_tile = kTileSizes[b->tp_index] - 1;
+    // the widest tiles, whatever the stages use: 127 cells for 128 threads
+    a.tiles = b->tiles[2];
+    a.ntiles = b->ntiles[2];
+    a.cells_per_tile = kTileSizes[2] - 1;
     a.gm1 = b->gamma - 1.0;
     a.gamma = b->gamma;
     a.cfl = cfl;
