@@ -882,6 +882,8 @@ static enomr_status rhs_with_epilogue(enomr_ctx *c, const double *U, const Epilo
         a.a = c->adv;
         a.inv_h = 1.0 / c->dx;
         a.speed = c->ax;
+        a.speed_next = nullptr;
+        a.status = c->status;
         a.sel = sel;
         a.epi = epi;
         prof_start(c, 1);
@@ -1220,6 +1222,45 @@ static enomr_status step_line(enomr_ctx *c, double *U, double dt, double cfl)
     return ENOMR_OK;
 }
 
+// One SSP-RK3 step of Burgers: the speed of U^n, the step, and three stages of
+// which the first two also take the speed of the state they make.  The last
+// stage's speed is left in c->ax.
+static enomr_status step_burgers(enomr_ctx *c, double *U, double dt, double cfl)
+{
+    if (!(dt > 0.0) && !(cfl > 0.0)) return ENOMR_EINVAL;
+    CU_TRY(cudaMemsetAsync(c->smax, 0, c->zero_bytes, c->stream));
+    double *speed[3] = {c->ax + 3, c->ax + 6, c->ax};
+    prof_start(c, 3);
+    cudaError_t e = launch_scalar_speed(U, c->nx, 1.0 / c->dx, speed[0], c->smax, c->status, c->stream);
+    prof_stop(c, 3);
+    CU_TRY(e);
+    CU_TRY(launch_set_dt(c->smax, cfl, dt > 0.0 ? dt : 0.0, c->dt, c->stream));
+    const double *from[3] = {U, c->U1, c->U2};
+    double *to[3] = {c->U1, c->U2, U};
+    for (int s = 0; s < 3; ++s) {
+        AdvArgs a;
+        memset(&a, 0, sizeof(a));
+        a.U = from[s];
+        a.n = c->nx;
+        a.bc = c->bc;
+        a.inv_h = 1.0 / c->dx;
+        a.speed = speed[s];
+        a.speed_next = s < 2 ? speed[s + 1] : nullptr;
+        a.status = c->status;
+        a.epi.mode = EPI_STAGE;
+        a.epi.c0 = RK_C0[s];
+        a.epi.c1 = RK_C1[s];
+        a.epi.dt_dev = c->dt;
+        a.epi.Un = U;
+        a.epi.out = to[s];
+        prof_start(c, 1);
+        e = by_order<BurgF>(c->order, a, c->stream);
+        prof_stop(c, 1);
+        CU_TRY(e);
+    }
+    return ENOMR_OK;
+}
+
 // One SSP-RK3 step of a short scalar line in one launch.
 static enomr_status step_small(enomr_ctx *c, double *U, double dt, double cfl)
 {
@@ -1254,8 +1295,9 @@ ENOMR_API enomr_status enomr_step(enomr_ctx *c, double *U, double dt, double cfl
     if (!c || !U) return ENOMR_EINVAL;
     const bool line = c->eq == ENOMR_EULER && c->ndim == 1;
     const bool small = c->eq != ENOMR_EULER && c->nx <= SMALL_CELLS;
-    if (line || small) {
-        enomr_status st = line ? step_line(c, U, dt, cfl) : step_small(c, U, dt, cfl);
+    if (line || small || c->eq == ENOMR_BURGERS) {
+        enomr_status st = line ? step_line(c, U, dt, cfl)
+                               : (small ? step_small(c, U, dt, cfl) : step_burgers(c, U, dt, cfl));
         if (st) return st;
         if (dt_used) {
             CU_TRY(cudaMemcpyAsync(dt_used, c->dt, sizeof(double), cudaMemcpyDeviceToHost,

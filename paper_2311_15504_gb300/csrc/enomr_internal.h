@@ -109,6 +109,8 @@ struct AdvArgs {
     int bc;
     double a, inv_h;
     const double *speed;   // Burgers: [max |u|, sign flags as bits] of U
+    double *speed_next;    // Burgers, optional: the same of the output, zeroed before
+    int *status;           // Burgers with speed_next: flags of the output's cells
     uint8_t *sel;          // optional [2][n+1]
     Epilogue epi;
 };

@@ -199,14 +199,45 @@ __global__ void __launch_bounds__(TP, SCALAR_CTAS) k_burgers(AdvArgs A)
         A.sel[A.n + 1 + k] = (uint8_t)selm;
     }
     __syncthreads();
+    unsigned long long m = 0, fl = 0;
     if (p < TP - 1) {
         const long long i = x0 + p;
         if (i < A.n) {
+            double o = 0.0;
             with_epilogue_form(A.epi, [&](auto M, auto P) {
-                epilogue_form<decltype(M)::value, decltype(P)::value != 0, false>(
+                o = epilogue_form<decltype(M)::value, decltype(P)::value != 0, false>(
                     A.epi, i, sFh[p + 1] - sFh[p], A.inv_h, A.U[i], false, 0.0);
             });
+            if (A.speed_next) {
+                const long long b = __double_as_longlong(o);
+                m = (unsigned long long)(b & 0x7fffffffffffffffLL);
+                fl = m == 0 ? 0 : ((b < 0) ? SGN_NEG : SGN_POS);
+                if (!below_1e300(o)) atomicOr(A.status, ST_NONPHYS_CELL);
+            }
         }
+    }
+    if (!A.speed_next) return;
+    // the next stage's speed and signs (k_scalar_speed): integer work only,
+    // which the FP64 pipe hides, instead of a launch that reads the state again
+    __shared__ unsigned long long red[TP / 32][2];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long x = __shfl_xor_sync(FULL, m, o);
+        m = m > x ? m : x;
+        fl |= __shfl_xor_sync(FULL, fl, o);
+    }
+    if ((p & 31) == 0) {
+        red[p >> 5][0] = m;
+        red[p >> 5][1] = fl;
+    }
+    __syncthreads();
+    if (p == 0) {
+        for (int w = 1; w < TP / 32; ++w) {
+            m = m > red[w][0] ? m : red[w][0];
+            fl |= red[w][1];
+        }
+        atomicMax((unsigned long long *)A.speed_next, m);
+        if (fl) atomicOr((unsigned long long *)(A.speed_next + 1), fl);
     }
 }
 

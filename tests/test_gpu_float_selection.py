@@ -64,12 +64,13 @@ def test_scalar_float_form(eq, order, n):
         s.check_status()
 
 
-@pytest.mark.parametrize("n", (18, 31, 32, 33, 200, 511, 512, 513, 1023, 1024, 1025))
+@pytest.mark.parametrize("n", (18, 31, 32, 33, 200, 511, 512, 513, 1023, 1024, 1025, 5000))
 @pytest.mark.parametrize("order", (5, 17))
 @pytest.mark.parametrize("eq", ("advection", "advection_left", "burgers", "burgers_left",
                                 "burgers_mixed"))
 def test_short_line_step_equals_its_stages(eq, order, n):
-    """enomr_step of at most 1024 cells is one launch; its stages are one each."""
+    """enomr_step of at most 1024 cells is one launch, a longer Burgers step takes
+    the next stage's speed in each stage; enomr_stage is one launch each."""
     from paper_2311_15504_gb300 import enomr
     h = 2.0 / n
     u = lines(n)["plateau"]
