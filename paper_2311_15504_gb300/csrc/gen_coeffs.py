@@ -211,6 +211,12 @@ def main(argv):
                 print("enomr_coeffs.h is stale", file=sys.stderr)
                 return 1
         return 0
+    # an unchanged header keeps its time stamp: the build compiles what is older
+    # than its newest header
+    if os.path.exists(path):
+        with open(path) as f:
+            if f.read() == text:
+                return 0
     with open(path, "w") as f:
         f.write(text)
     return 0
