@@ -48,12 +48,17 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
     __shared__ double sF[C][NL][S];
     __shared__ double sP[4][NL][S];  // sqrt(rho), u_n, u_t, H
     __shared__ double sLb[C][NL][TP + 1];
-    __shared__ double sWB[NL][TP][2 * g];
-    __shared__ double sQB[NL][TP][2 * g];
+    // per interface: the cotangents of a field's window; after the fields, G
+    __shared__ union {
+        struct {
+            double d[NL][TP][2 * g], q[NL][TP][2 * g];
+        } w;
+        double G[NL][TP][2 * C];
+    } sW;
+    static_assert(2 * C <= 4 * g, "G fits in the windows' storage");
     __shared__ double sRow[NL][TP][3];
     __shared__ double sRowA[NL][TP][4];
     __shared__ double sRoeB[NL][TP][2][C];
-    __shared__ double sG[NL][TP][2 * C];
     __shared__ double sA[T * W];
 
     const long long nx = A.nx, ny = A.ny, ncell = nx * ny;
@@ -160,20 +165,17 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
     // sides.  A field with that choice (nearly all in smooth flow) has its sums
     // over the window, and its part of the cells' cotangents, in common with the
     // others up to factors of the field: X and Y once instead of eight sums per
-    // field, and one gather of G (below) instead of one per field.  What the
-    // windows on other choices differ by goes through the per-field path.  (FP64
-    // pipe bound: about half the operations.  Vortex with weak waves, 512^2,
-    // order 9, rollout of two steps and its gradient: 16.1 -> 13.1 ms.)
+    // field, and one gather of G (below) instead of one per field.  A field on
+    // another choice takes no part in it and goes through the per-field path
+    // whole, so that no cell outside its stencils enters.  Both parts are left
+    // out where nothing needs them: the sums by warps, the gathers by CTAs.
+    // (FP64 pipe bound.  One transposed product, order 9, 512^2: smooth periodic
+    // flow 1.95 -> 1.36 ms with the common part; four-quadrant Riemann state,
+    // hardly any full stencil, 1.91 / 1.98 ms.)
     double X[C], Y[C], GU[C], GF[C];
+    bool have = false;  // X and Y are set
 #pragma unroll
-    for (int q = 0; q < C; ++q) {
-        X[q] = Y[q] = GU[q] = GF[q] = 0.0;
-#pragma unroll
-        for (int j = 0; j < 2 * g; ++j) {
-            X[q] = fma(Coef<R>::m()[j], sU[q][line][p + j], X[q]);
-            Y[q] = fma(Coef<R>::p()[j], sF[q][line][p + j], Y[q]);
-        }
-    }
+    for (int q = 0; q < C; ++q) X[q] = Y[q] = GU[q] = GF[q] = 0.0;
 
     double ftv[C];
     double hq_b = 0.0, uh_b = 0.0, vh_b = 0.0, kap_b = 0.0, c2g_b = 0.0;
@@ -257,10 +259,29 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
         // w_bar = alpha d and q_bar = P + M; the sums S[q] = sum_j d_j U_j[q]
         // give both the U part of the row-coefficient cotangents (alpha S) and
         // the alpha cotangent sum_j d_j w_j = l . S.
-        double S0 = ftb * X[0], S1 = ftb * X[1], ST = C == 4 ? ftb * X[2 % C] : 0.0,
-               SE = ftb * X[C - 1];
-        double Q0 = ftb * Y[0], Q1 = ftb * Y[1], QT = C == 4 ? ftb * Y[2 % C] : 0.0;
-        {
+        const bool full = (selp | selm) == 0;
+        const bool other = owned && !full;
+        if (!have && __any_sync(FULL, owned && full)) {
+            have = true;
+#pragma unroll
+            for (int q = 0; q < C; ++q)
+#pragma unroll
+                for (int j = 0; j < 2 * g; ++j) {
+                    X[q] = fma(Coef<R>::m()[j], sU[q][line][p + j], X[q]);
+                    Y[q] = fma(Coef<R>::p()[j], sF[q][line][p + j], Y[q]);
+                }
+        }
+        double S0 = 0.0, S1 = 0.0, ST = 0.0, SE = 0.0, Q0 = 0.0, Q1 = 0.0, QT = 0.0;
+        if (owned && full) {
+            S0 = ftb * X[0];
+            S1 = ftb * X[1];
+            SE = ftb * X[C - 1];
+            Q0 = ftb * Y[0];
+            Q1 = ftb * Y[1];
+            if (C == 4) {
+                ST = ftb * X[2 % C];
+                QT = ftb * Y[2 % C];
+            }
             const double fa = ftb * alpha;
             GU[0] = fma(fa, l0c, GU[0]);
             GF[0] = fma(ftb, l0c, GF[0]);
@@ -278,10 +299,9 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
                 }
             }
         }
-        const bool other = owned && (selp | selm) != 0;
         const bool others = __syncthreads_or(other) != 0;
         if (others) {
-            // the frozen choice's weights minus the full stencil's, times ftb
+            // the frozen choice's weights, times ftb
             constexpr int c0 = g - 1;
             double wp[W], wm[W];
 #pragma unroll
@@ -299,8 +319,8 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
                     a = selp == T + 1 ? -0.5 : a;
                     b = selm == T + 1 ? -0.5 : b;
                 }
-                wp[j] = other ? (a - sA[j]) * ftb : 0.0;
-                wm[j] = other ? (b - sA[j]) * ftb : 0.0;
+                wp[j] = other ? a * ftb : 0.0;
+                wm[j] = other ? b * ftb : 0.0;
             }
 #pragma unroll
             for (int j = 0; j < 2 * g; ++j) {
@@ -308,8 +328,8 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
                 const double P = (j <= 2 * g - 2) ? wp[j] : 0.0;
                 const double M = (j >= 1) ? wm[2 * g - 1 - j] : 0.0;
                 const double qb = P + M, d = P - M;
-                sWB[line][p][j] = d;  // alpha is folded into the gather's row
-                sQB[line][p][j] = qb;
+                sW.w.d[line][p][j] = d;  // alpha is folded into the gather's row
+                sW.w.q[line][p][j] = qb;
                 S0 = fma(d, sU[0][line][s], S0);
                 Q0 = fma(qb, sF[0][line][s], Q0);
                 if (C == 4) ST = fma(d, sU[2][line][s], ST);
@@ -335,13 +355,13 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
         }
         // gather rows: U part scaled by alpha (it multiplies d), F part not
         if (others) {
-        sRow[line][p][0] = l0c;
-        sRow[line][p][1] = l1c;
-        sRow[line][p][2] = (C == 4) ? -vh : 0.0;
-        sRowA[line][p][0] = alpha * l0c;
-        sRowA[line][p][1] = alpha * l1c;
-        sRowA[line][p][2] = (C == 4) ? -alpha * vh : 0.0;
-        sRowA[line][p][3] = alpha;
+            sRow[line][p][0] = l0c;
+            sRow[line][p][1] = l1c;
+            sRow[line][p][2] = (C == 4) ? -vh : 0.0;
+            sRowA[line][p][0] = alpha * l0c;
+            sRowA[line][p][1] = alpha * l1c;
+            sRowA[line][p][2] = (C == 4) ? -alpha * vh : 0.0;
+            sRowA[line][p][3] = alpha;
         }
         // row coefficients -> Roe scalars
         if (shear) {
@@ -380,7 +400,7 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
                 for (int j = 0; j < 2 * g; ++j) {
                     const int pp = s - j;
                     if (pp < 0 || pp >= TP) continue;
-                    const double d = sWB[gl][pp][j], qb = sQB[gl][pp][j];
+                    const double d = sW.w.d[gl][pp][j], qb = sW.w.q[gl][pp][j];
                     const double r0 = sRow[gl][pp][0], a0 = sRowA[gl][pp][0];
                     const double al_ = sRowA[gl][pp][3];
                     if (shear) {
@@ -412,12 +432,12 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
     // weight of its place in the window of interface p' = s - j times G
 #pragma unroll
     for (int q = 0; q < C; ++q) {
-        sG[line][p][q] = GU[q];
-        sG[line][p][C + q] = GF[q];
+        sW.G[line][p][q] = GU[q];
+        sW.G[line][p][C + q] = GF[q];
     }
-    __syncthreads();
+    const bool common = __syncthreads_or(have) != 0;
 #pragma unroll
-    for (int c = 0; c < CPT; ++c) {
+    for (int c = 0; c < CPT && common; ++c) {
         const int idx = tid + c * NT;
         if (idx < NL * S) {
             int gl, s;
@@ -434,8 +454,8 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
                 if (pp < 0 || pp >= TP) continue;
 #pragma unroll
                 for (int q = 0; q < C; ++q) {
-                    cUb[c][q] = fma(Coef<R>::m()[j], sG[gl][pp][q], cUb[c][q]);
-                    cFb[c][q] = fma(Coef<R>::p()[j], sG[gl][pp][C + q], cFb[c][q]);
+                    cUb[c][q] = fma(Coef<R>::m()[j], sW.G[gl][pp][q], cUb[c][q]);
+                    cFb[c][q] = fma(Coef<R>::p()[j], sW.G[gl][pp][C + q], cFb[c][q]);
                 }
             }
         }
