@@ -111,8 +111,9 @@ __global__ void __launch_bounds__(256, 5) k_alpha(AlphaArgs A)
     const long long ncell = A.nx * A.ny;
     if (C == 4 && A.dead_a && blockIdx.x > 0 && blockIdx.y > 0) {
         // This state was combined from two others.  Where this block and all
-        // around it are dead in both, they hold one state here too: no cell is
-        // a representative, and nothing is read.
+        // around it are dead in both, they hold one state here too (a mean of
+        // the two, in range as they are): no cell is a representative, and
+        // nothing is read.
         bool dead = true;
         if (tid < 9) {
             const int bx = (int)blockIdx.x + tid % 3 - 1, by = (int)blockIdx.y + tid / 3 - 1;
@@ -199,7 +200,9 @@ __global__ void __launch_bounds__(256, 5) k_alpha(AlphaArgs A)
         }
     }
     if (C == 4 && A.flat) {
-        const bool any = __syncthreads_or(differs) != 0;
+        // one state, and its flux is a number: F - F of equal cells is 0 then
+        // (thread 0 holds the block's first cell)
+        const bool any = __syncthreads_or(differs || (tid == 0 && !ordinary_state<C>(ur[0]))) != 0;
         if (tid == 0) A.flat[(long long)blockIdx.y * gridDim.x + blockIdx.x] = !any;
     } else {
         __syncthreads();

@@ -20,6 +20,21 @@ __device__ __forceinline__ bool below_1e300(double x)
     return (__double_as_longlong(x) & 0x7fffffffffffffffLL) < 0x7e37e43c8800759cLL;
 }
 
+// Whether the Euler fluxes of state u are finite, from the exponents alone (no
+// FP64 work): density in [2^-100, 2^240), momenta and energy below 2^240, so
+// that velocities stay below 2^340, pressure below 2^600 and (E + p) u below
+// 2^1000.  States outside that have finite fluxes too, or not: false.
+template <int C>
+__device__ __forceinline__ bool ordinary_state(const double *u)
+{
+    const unsigned rho = (unsigned)__double2hiint(u[0]) >> 20;  // with the sign: a negative one fails
+    bool ok = rho >= 1023u - 100u && rho < 1023u + 240u;
+#pragma unroll
+    for (int q = 1; q < C; ++q)
+        ok = ok && (((unsigned)__double2hiint(u[q]) >> 20) & 0x7ffu) < 1023u + 240u;
+    return ok;
+}
+
 // The step of a state whose CFL speed is sm.
 __device__ __forceinline__ double step_size(double sm, double cfl, double dt_fixed)
 {

@@ -48,13 +48,14 @@ struct SideDev {
     double st_lo[4], st_hi[4];
 };
 
-// Map of the cell blocks of a 2D state that hold one state together with all
-// the blocks around them ("dead" blocks: every flux difference of their cells
-// is exactly zero), and the lists made from it: the tiles of both sweeps that
-// touch another block, and the dead blocks.
+// Map of the cell blocks of a 2D state that hold one state of finite flux
+// together with all the blocks around them ("dead" blocks: every flux
+// difference of their cells is exactly zero), and the lists made from it: the
+// tiles of both sweeps that touch another block, and the dead blocks.
 constexpr int MAP_B = 32;  // cells per block side; at least the widest halo, 9
 struct TileMap {
-    const unsigned char *flat;  // [nby][nbx]: every cell equals its left and upper neighbour
+    const unsigned char *flat;  // [nby][nbx]: every cell equals its left and upper neighbour,
+                                // and the first one's flux is finite (ordinary_state)
     unsigned char *dead;        // [nby][nbx]
     int nbx, nby;
     long long nx, ny;
