@@ -25,7 +25,15 @@
 namespace enomr {
 
 constexpr int LINE_TP = 32, LINE_THREADS = 192;
-constexpr long long LINE_MAX_CELLS = 1LL << 17;
+
+// Longest line that runs here; above, where the chip is full, k_sweep, which
+// forms a window's projections once for both sides.  A step on the shock /
+// entropy wave, this over k_sweep (the same with random cells): order 9, 20 000
+// cells 0.81 (0.72), 40 000 0.99 (1.00), 65 000 1.10 (1.22), 131 072 1.17
+// (1.22); order 5 0.85, 0.97, 1.09, 1.16; order 11, 40 000 0.84 (0.86), 65 000
+// 0.99 (1.03), 100 000 1.15 (1.19); order 17 0.75 (0.84), 0.92 (0.98), 1.06 (1.13).
+template <int R>
+constexpr long long LINE_MAX_CELLS = R <= 9 ? 40000 : 65000;
 
 template <int R>
 __global__ void __launch_bounds__(LINE_THREADS) k_line(SweepArgs A)

@@ -28,13 +28,9 @@ template <int R> cudaError_t launch_burgers(const AdvArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// k_line up to 2^17 cells; above, where the chip is full, k_sweep, which forms
-// a window's projections once for both sides: order 9, 100 000 cells, 143
-// against 125 us a launch, but 25 000 cells 48 against 48, 6400 cells 23
-// against 42, 400 cells 18 against 41.
 template <int R> cudaError_t launch_euler1d(const SweepArgs &a, cudaStream_t s)
 {
-    if (a.nx <= LINE_MAX_CELLS) return launch_line<R>(a, s);
+    if (a.nx <= LINE_MAX_CELLS<R>) return launch_line<R>(a, s);
     const long long tiles = (a.nx + E1_TP - 2) / (E1_TP - 1);
     k_sweep<R, 3, 0, E1_TP, 1><<<dim3((unsigned)tiles, 1), E1_TP, 0, s>>>(a);
     return cudaGetLastError();

@@ -1,7 +1,7 @@
 """The single-problem 1D Euler step against the batched one, bit for bit.
 
-enomr_step on a line runs the window-per-warp sweep (tiles of 31 cells; above
-2^17 cells the interface-per-lane one) with the next stage's wave speeds in its
+enomr_step on a line runs the window-per-warp sweep (tiles of 31 cells; on long
+lines the interface-per-lane one) with the next stage's wave speeds in its
 epilogue; the batch runs its own tile function and reductions.
 """
 import numpy as np
@@ -65,3 +65,10 @@ def test_fixed_step_equals_its_stages():
     s.step(v, dt)
     assert torch.equal(a, v)
     s.check_status()
+
+
+@pytest.mark.parametrize("order, longest", ((5, 40000), (9, 40000), (11, 65000), (17, 65000)))
+def test_lines_beside_the_change_of_sweep_equal_batch(order, longest):
+    """The longest line that the window-per-warp sweep takes, and one cell more."""
+    for bc in (0, 1):
+        compare([longest, longest + 1], order, bc, 2)
