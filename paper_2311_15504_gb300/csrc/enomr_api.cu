@@ -736,8 +736,8 @@ static enomr_status cu(cudaError_t e) { return e == cudaSuccess ? ENOMR_OK : ENO
 
 static int valid_order(int R) { return R >= 5 && R <= 17 && (R % 2) == 1; }
 
-// Block map slots: U^n, U^(1), U^(2) of a step; MAP_NONE: none is made.
-enum : int { MAP_NONE = -1, MAP_N = 0, MAP_1 = 1, MAP_2 = 2 };
+// Block map slots: 0, 1, 2 for U^n, U^(1), U^(2) of a step; MAP_NONE: none is made.
+enum : int { MAP_NONE = -1, MAP_N = 0 };
 
 static long long map_blocks(const enomr_ctx *c)
 {

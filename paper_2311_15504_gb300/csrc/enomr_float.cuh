@@ -1,5 +1,5 @@
 // enomr_float.cuh -- floats of doubles on the integer ALU, and the bounds of
-// the float form of the selection (enomr_select.cuh, mr_select).
+// the float form of the selection (select_float, mr_select).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -49,21 +49,17 @@ __host__ __device__ constexpr float binomial(int n, int k)
     return (float)r;  // at most C(15, 7) = 6435: exact
 }
 
-// Bound units.  EPS: relative error of a difference e_j against its
-// magnitude m_j, in 2^-24 (scalar: the truncation to float, m_j = |e_j|).
-// OPS: FP64 roundings of a window value.
-template <int EPS, int OPS>
-struct SelBound {
-    // K terms: K fused products, one rounding each
-    __host__ __device__ static constexpr float terms(int K) { return 0x1p-24f * (EPS + K + 2); }
-    // FP64 evaluation of an indicator of order K: the roundings of the values
-    // times sum |b| = 2^K, and one rounding per term of the partial sums of
-    // alternating binomials, +-C(K-1, i) times the centre value up to terms
-    // of the size of the differences: 2^(K-1) in all
-    __host__ __device__ static constexpr float values(int K)
-    {
-        return 0x1.1p-53f * (float)(1 << K) * (OPS + 0.5f);
-    }
-};
+// Bounds of the float form of an indicator of order K = m + n against the value
+// that the FP64 evaluation compares: float_error(K) * sum |b'_j| |e_j| +
+// fp64_error(K) * |v_c|.
+
+// K fused products, one rounding each, of differences truncated to float (twice
+// 2^-24), and the final additions
+__host__ __device__ constexpr float float_error(int K) { return 0x1p-24f * (float)(K + 4); }
+
+// the FP64 evaluation: one rounding per term of the partial sums of alternating
+// binomials, +-C(K-1, i) times the centre value up to terms of the size of the
+// differences: 2^(K-1) in all
+__host__ __device__ constexpr float fp64_error(int K) { return 0x1.1p-54f * (float)(1 << K); }
 
 }  // namespace enomr

@@ -108,9 +108,9 @@ __device__ __forceinline__ void mr_select64(const double *v, bool valid, int &se
 }
 
 // The same selection from the differences e_j = v_{j+1} - v_j in float, each
-// comparison with a bound on its distance from the FP64 values' (SelBound);
-// windows that it leaves open are selected in FP64, so the outcome is that of
-// mr_select64 always.  FP64 work: 2g - 2 subtractions instead of 6 + m + n + 1
+// comparison with a bound on its distance from the FP64 values' (float_error,
+// fp64_error); windows that it leaves open are selected in FP64, so the outcome
+// is that of mr_select64 always.  FP64 work: 2g - 2 subtractions instead of 6 + m + n + 1
 // operations for every candidate that is tested (10 to 26 of them at a front,
 // orders 9 to 17); the FP32 pipe does 64 operations in the time of one of
 // those.  The walk is a loop over the coefficient table (constant operands,
@@ -120,15 +120,14 @@ template <int R>
 __device__ __forceinline__ void mr_select(const double *v, bool valid, int &sel)
 {
     constexpr int g = (R + 1) / 2, T = Tab<R>::T, c = g - 1, N = 2 * g - 2;
-    using B = SelBound<2, 0>;
     float e[N];
 #pragma unroll
     for (int j = 0; j < N; ++j) e[j] = to_float(v[j + 1] - v[j]);
     const float S = fabsf(to_float(v[c]));
     const bool none = (e[c - 1] == 0.0f && e[c - 2] == 0.0f) || (e[c] == 0.0f && e[c + 1] == 0.0f);
-    const float al = fabsf(e[c - 1]), ar = fabsf(e[c]), sv = S * B::values(2);
-    const float el = __fmaf_rn(al + fabsf(e[c - 2]), B::terms(2), sv);
-    const float er = __fmaf_rn(ar + fabsf(e[c + 1]), B::terms(2), sv);
+    const float al = fabsf(e[c - 1]), ar = fabsf(e[c]), sv = S * fp64_error(2);
+    const float el = __fmaf_rn(al + fabsf(e[c - 2]), float_error(2), sv);
+    const float er = __fmaf_rn(ar + fabsf(e[c + 1]), float_error(2), sv);
     const float L = fmaxf(al, fabsf(e[c - 1] - e[c - 2])), Q = fmaxf(ar, fabsf(e[c + 1] - e[c]));
     const float lo = fminf(L - el, Q - er), hi = fminf(L + el, Q + er);
     bool open = !(S <= 0x1p90f) || !(el + er <= 0x1p90f);  // NaN, out of range
@@ -144,8 +143,7 @@ __device__ __forceinline__ void mr_select(const double *v, bool valid, int &sel)
             a = __fmaf_rn(fabsf(b), fabsf(e[j]), a);
         }
         const int K = Coef<R>::order(t);
-        const float err = __fmaf_rn(a, 0x1p-24f * (float)(K + 4),
-                                    S * (B::values(0) * __int_as_float((127 + K) << 23)));
+        const float err = __fmaf_rn(a, float_error(K), S * fp64_error(K));
         s = fabsf(s);
         if (active && s + err < lo) {
             sel = t;
@@ -160,7 +158,7 @@ __device__ __forceinline__ void mr_select(const double *v, bool valid, int &sel)
         open = false;
     } else if (active) {
         // minmod(f_{j+1} - f_j, f_j - f_{j-1})
-        const float e1 = __fmaf_rn(al, B::terms(2), sv), e2 = __fmaf_rn(ar, B::terms(2), sv);
+        const float e1 = __fmaf_rn(al, float_error(2), sv), e2 = __fmaf_rn(ar, float_error(2), sv);
         if (!(al > e1) || !(ar > e2))
             open = true;
         else if ((e[c - 1] < 0.0f) != (e[c] < 0.0f))

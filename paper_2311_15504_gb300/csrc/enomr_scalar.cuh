@@ -23,7 +23,6 @@ __device__ __forceinline__ double scalar_value(const double *v0, const float2 *e
                                                int &sel)
 {
     constexpr int g = (R + 1) / 2, W = 2 * g - 1, T = Tab<R>::T, c = g - 1, N = W - 1;
-    using B = SelBound<2, 0>;
     float e[N];
     float emax = 0.0f;
 #pragma unroll
@@ -34,7 +33,7 @@ __device__ __forceinline__ double scalar_value(const double *v0, const float2 *e
     const float vc = fabsf(to_float(v0[DIRN * c]));
     const bool left0 = e[c - 1] == 0.0f && e[c - 2] == 0.0f;
     const bool right0 = e[c] == 0.0f && e[c + 1] == 0.0f;
-    sel = select_float<R, B, false>(e, e, vc, left0, right0);
+    sel = select_float<R>(e, vc, left0, right0);
     const bool open = valid && sel == SEL_OPEN;
     if (__any_sync(FULL, open)) {
         double v[W];

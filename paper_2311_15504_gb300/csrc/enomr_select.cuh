@@ -54,60 +54,51 @@ struct PairSum {
 // Largest |e_j| over |v_c| for which the pair sum is taken.
 constexpr float PAIR_RANGE = 0x1p-6f;
 
-template <int R, int t, class B, bool REV>
-__device__ __forceinline__ void select_walk(const float *e, const float *m, float S, float lo,
-                                            float hi, int &sel)
+template <int R, int t>
+__device__ __forceinline__ void select_walk(const float *e, float S, float lo, float hi, int &sel)
 {
-    constexpr int g = (R + 1) / 2, c = g - 1, N = 2 * g - 2, T = Tab<R>::T;
+    constexpr int g = (R + 1) / 2, c = g - 1, T = Tab<R>::T;
     if constexpr (t < T) {
         constexpr int K = Cand<R, t>::m + Cand<R, t>::n, j0 = c - Cand<R, t>::m;
         float s = 0.0f, a = 0.0f;
 #pragma unroll
         for (int i = 0; i < K; ++i) {
             const float b = ((K - 1 - i) & 1) ? -binomial(K - 1, i) : binomial(K - 1, i);
-            const int j = REV ? N - 1 - (j0 + i) : j0 + i;
-            s = i == 0 ? __fmul_rn(b, e[j]) : __fmaf_rn(b, e[j], s);
-            a = i == 0 ? fabsf(b) * fabsf(m[j]) : __fmaf_rn(fabsf(b), fabsf(m[j]), a);
+            s = i == 0 ? __fmul_rn(b, e[j0 + i]) : __fmaf_rn(b, e[j0 + i], s);
+            a = i == 0 ? fabsf(b) * fabsf(e[j0 + i]) : __fmaf_rn(fabsf(b), fabsf(e[j0 + i]), a);
         }
-        const float err = __fmaf_rn(a, B::terms(K), S * B::values(K));
+        const float err = __fmaf_rn(a, float_error(K), S * fp64_error(K));
         s = fabsf(s);
         if (s + err < lo) {
             sel = t;
         } else if (s - err > hi) {
-            select_walk<R, t + 1, B, REV>(e, m, S, lo, hi, sel);
+            select_walk<R, t + 1>(e, S, lo, hi, sel);
         } else {
             sel = SEL_OPEN;
         }
     }
 }
 
-// Selection of the window with differences e_j (j = 0 .. 2g-3) and their
-// magnitudes m_j >= the size of the terms that formed e_j; S: bound of the
-// size of the terms that formed the centre value.  REV: e and m run against
-// the window (window difference i is entry 2g-3-i; the sign of all of them
-// is immaterial).  left0, right0: the three cells ending / starting at the
+// Selection of the window with differences e_j (j = 0 .. 2g-3); S: size of the
+// centre value.  left0, right0: the three cells ending / starting at the
 // centre are bitwise equal.  Returns 0 .. T+2 or SEL_OPEN.
-template <int R, class B, bool REV>
-__device__ __forceinline__ int select_float(const float *e, const float *m, float S, bool left0,
-                                            bool right0)
+template <int R>
+__device__ __forceinline__ int select_float(const float *e, float S, bool left0, bool right0)
 {
-    constexpr int g = (R + 1) / 2, c = g - 1, N = 2 * g - 2, T = Tab<R>::T;
+    constexpr int g = (R + 1) / 2, c = g - 1, T = Tab<R>::T;
     if (left0 || right0) return T + 2;  // IS_0 = 0: no candidate passes, minmod(a, b) = 0
-    auto at = [&](const float *p, int j) { return p[REV ? N - 1 - j : j]; };
-    const float l1 = at(e, c - 1), l2 = at(e, c - 2), r1 = at(e, c), r2 = at(e, c + 1);
-    const float ml = fabsf(at(m, c - 1)), mr = fabsf(at(m, c));
-    const float sv = S * B::values(2);
-    const float el = __fmaf_rn(ml + fabsf(at(m, c - 2)), B::terms(2), sv);
-    const float er = __fmaf_rn(mr + fabsf(at(m, c + 1)), B::terms(2), sv);
-    const float L = fmaxf(fabsf(l1), fabsf(l1 - l2)), Q = fmaxf(fabsf(r1), fabsf(r2 - r1));
+    const float l1 = e[c - 1], l2 = e[c - 2], r1 = e[c], r2 = e[c + 1];
+    const float al = fabsf(l1), ar = fabsf(r1), sv = S * fp64_error(2);
+    const float el = __fmaf_rn(al + fabsf(l2), float_error(2), sv);
+    const float er = __fmaf_rn(ar + fabsf(r2), float_error(2), sv);
+    const float L = fmaxf(al, fabsf(l1 - l2)), Q = fmaxf(ar, fabsf(r2 - r1));
     const float lo = fminf(L - el, Q - er), hi = fminf(L + el, Q + er);
     int sel = T;
     if (!(S <= 0x1p90f) || !(el + er <= 0x1p90f)) return SEL_OPEN;  // NaN or out of range
-    select_walk<R, 0, B, REV>(e, m, S, lo, hi, sel);
+    select_walk<R, 0>(e, S, lo, hi, sel);
     if (sel != T) return sel;
     // every candidate failed: minmod(f_{j+1} - f_j, f_j - f_{j-1})
-    const float e1 = __fmaf_rn(ml, B::terms(2), sv), e2 = __fmaf_rn(mr, B::terms(2), sv);
-    const float al = fabsf(l1), ar = fabsf(r1);
+    const float e1 = __fmaf_rn(al, float_error(2), sv), e2 = __fmaf_rn(ar, float_error(2), sv);
     if (!(al > e1) || !(ar > e2)) return SEL_OPEN;
     if ((l1 < 0.0f) != (r1 < 0.0f)) return T + 2;
     if (ar + e2 < al - e1) return T;
