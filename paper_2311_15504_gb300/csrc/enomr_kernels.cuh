@@ -89,7 +89,7 @@ __device__ __forceinline__ void mr_select64(const double *v, bool valid, int &se
     // Step 1, Eq. (Baseline_IS)
     const double d1L = v[c] - v[c - 1];
     const double d2L = fma(-2.0, v[c - 1], v[c]) + v[c - 2];
-    const double d1R = v[c] - v[c + 1];
+    const double d1R = -(v[c + 1] - v[c]);
     const double d2R = fma(-2.0, v[c + 1], v[c]) + v[c + 2];
     const long long is0 = imin64(imax64(abits(d1L), abits(d2L)), imax64(abits(d1R), abits(d2R)));
     // IS >= 0 always, so with IS_0 = 0 no candidate can pass: skip the walk
@@ -107,70 +107,95 @@ __device__ __forceinline__ void mr_select64(const double *v, bool valid, int &se
     }
 }
 
+// Windows whose cells lie within this many ulp of the centre's are constant up to
+// rounding: the bound of the FP64 evaluation of the widest indicator (fp64_error)
+// is about that large, so that no candidate can pass in float.
+template <int R>
+constexpr unsigned long long NOISE_ULP = R <= 9 ? 64 : 1ULL << (R - 3);
+
 // The same selection from the differences e_j = v_{j+1} - v_j in float, each
 // comparison with a bound on its distance from the FP64 values' (float_error,
 // fp64_error); windows that it leaves open are selected in FP64, so the outcome
-// is that of mr_select64 always.  FP64 work: 2g - 2 subtractions instead of 6 + m + n + 1
-// operations for every candidate that is tested (10 to 26 of them at a front,
-// orders 9 to 17); the FP32 pipe does 64 operations in the time of one of
+// is that of mr_select64 always.  FP64 work: 2g - 2 subtractions instead of 6 +
+// m + n + 1 operations for every candidate that is tested (10 to 26 of them at a
+// front, orders 9 to 17); the FP32 pipe does 64 operations in the time of one of
 // those.  The walk is a loop over the coefficient table (constant operands,
 // one candidate at a time for the whole warp) to keep the code small: the
 // sweeps hold several copies of it.
+// A warp of which every window is constant up to rounding (or exactly) goes to
+// FP64 without the float form, which would be left open there and only add to
+// it; integer work alone decides that.  Cells equal to within 8 ulp, a launch
+// with the float form tried everywhere / now / FP64 alone: 64^2, order 17, 478 /
+// 449 / 413 us; 1D, 300 000 cells, order 17, 1485 / 1453 / 1439 us.  Per lane or
+// for any such window of a warp the rule is the slower one at fronts, whose other
+// lanes the float form decides (2048^2 Riemann state, order 17, a step 3.67 ->
+// 4.04 ms).
 template <int R>
 __device__ __forceinline__ void mr_select(const double *v, bool valid, int &sel)
 {
     constexpr int g = (R + 1) / 2, T = Tab<R>::T, c = g - 1, N = 2 * g - 2;
-    float e[N];
+    bool open = valid, noise = true;
 #pragma unroll
-    for (int j = 0; j < N; ++j) e[j] = to_float(v[j + 1] - v[j]);
-    const float S = fabsf(to_float(v[c]));
-    const bool none = (e[c - 1] == 0.0f && e[c - 2] == 0.0f) || (e[c] == 0.0f && e[c + 1] == 0.0f);
-    const float al = fabsf(e[c - 1]), ar = fabsf(e[c]), sv = S * fp64_error(2);
-    const float el = __fmaf_rn(al + fabsf(e[c - 2]), float_error(2), sv);
-    const float er = __fmaf_rn(ar + fabsf(e[c + 1]), float_error(2), sv);
-    const float L = fmaxf(al, fabsf(e[c - 1] - e[c - 2])), Q = fmaxf(ar, fabsf(e[c + 1] - e[c]));
-    const float lo = fminf(L - el, Q - er), hi = fminf(L + el, Q + er);
-    bool open = !(S <= 0x1p90f) || !(el + er <= 0x1p90f);  // NaN, out of range
-    sel = valid ? T : 0;
-    bool active = valid && !none && !open;
+    for (int j = c - 2; j <= c + 2; ++j) {
+        const unsigned long long d = (unsigned long long)__double_as_longlong(v[j]) -
+                                     (unsigned long long)__double_as_longlong(v[c]);
+        noise = noise && d + NOISE_ULP<R> <= 2 * NOISE_ULP<R>;
+    }
+    if (!__all_sync(FULL, noise || !valid)) {
+        float e[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) e[j] = to_float(v[j + 1] - v[j]);
+        const float S = fabsf(to_float(v[c]));
+        const bool none = (e[c - 1] == 0.0f && e[c - 2] == 0.0f) || (e[c] == 0.0f && e[c + 1] == 0.0f);
+        const float al = fabsf(e[c - 1]), ar = fabsf(e[c]), sv = S * fp64_error(2);
+        const float el = __fmaf_rn(al + fabsf(e[c - 2]), float_error(2), sv);
+        const float er = __fmaf_rn(ar + fabsf(e[c + 1]), float_error(2), sv);
+        const float L = fmaxf(al, fabsf(e[c - 1] - e[c - 2])), Q = fmaxf(ar, fabsf(e[c + 1] - e[c]));
+        const float lo = fminf(L - el, Q - er), hi = fminf(L + el, Q + er);
+        open = !(S <= 0x1p90f) || !(el + er <= 0x1p90f);  // NaN, out of range
+        sel = valid ? T : 0;
+        bool active = valid && !none && !open;
 #pragma unroll 1
-    for (int t = 0; t < T && __any_sync(FULL, active); ++t) {
-        float s = 0.0f, a = 0.0f;
+        for (int t = 0; t < T && __any_sync(FULL, active); ++t) {
+            float s = 0.0f, a = 0.0f;
 #pragma unroll
-        for (int j = 0; j < N; ++j) {
-            const float b = Coef<R>::e()[t * N + j];
-            s = __fmaf_rn(b, e[j], s);
-            a = __fmaf_rn(fabsf(b), fabsf(e[j]), a);
+            for (int j = 0; j < N; ++j) {
+                const float b = Coef<R>::e()[t * N + j];
+                s = __fmaf_rn(b, e[j], s);
+                a = __fmaf_rn(fabsf(b), fabsf(e[j]), a);
+            }
+            const int K = Coef<R>::order(t);
+            const float err = __fmaf_rn(a, float_error(K), S * fp64_error(K));
+            s = fabsf(s);
+            if (active && s + err < lo) {
+                sel = t;
+                active = false;
+            } else if (active && !(s - err > hi)) {
+                open = true;
+                active = false;
+            }
         }
-        const int K = Coef<R>::order(t);
-        const float err = __fmaf_rn(a, float_error(K), S * fp64_error(K));
-        s = fabsf(s);
-        if (active && s + err < lo) {
-            sel = t;
-            active = false;
-        } else if (active && !(s - err > hi)) {
-            open = true;
-            active = false;
+        if (none) {
+            if (valid) sel = T + 2;  // IS_0 = 0: no candidate passes, minmod(a, b) = 0
+            open = false;
+        } else if (active) {
+            // minmod(f_{j+1} - f_j, f_j - f_{j-1})
+            const float e1 = __fmaf_rn(al, float_error(2), sv), e2 = __fmaf_rn(ar, float_error(2), sv);
+            if (!(al > e1) || !(ar > e2))
+                open = true;
+            else if ((e[c - 1] < 0.0f) != (e[c] < 0.0f))
+                sel = T + 2;
+            else if (ar + e2 < al - e1)
+                sel = T;
+            else if (al + e1 < ar - e2)
+                sel = T + 1;
+            else
+                open = true;
         }
+        open = open && valid;
+    } else {
+        sel = 0;
     }
-    if (none) {
-        if (valid) sel = T + 2;  // IS_0 = 0: no candidate passes, minmod(a, b) = 0
-        open = false;
-    } else if (active) {
-        // minmod(f_{j+1} - f_j, f_j - f_{j-1})
-        const float e1 = __fmaf_rn(al, float_error(2), sv), e2 = __fmaf_rn(ar, float_error(2), sv);
-        if (!(al > e1) || !(ar > e2))
-            open = true;
-        else if ((e[c - 1] < 0.0f) != (e[c] < 0.0f))
-            sel = T + 2;
-        else if (ar + e2 < al - e1)
-            sel = T;
-        else if (al + e1 < ar - e2)
-            sel = T + 1;
-        else
-            open = true;
-    }
-    open = open && valid;
     if (__any_sync(FULL, open)) {
         int s64;
         mr_select64<R>(v, open, s64);
@@ -195,10 +220,8 @@ __device__ __forceinline__ double mr_recon(const double *v, const double *sA, in
 #pragma unroll
         for (int l = 0; l < W; ++l) val = fma(row[l], v[l], val);
     } else {
-        double mm = 0.0;
-        if (sel == T) mm = -(v[c] - v[c + 1]);
-        if (sel == T + 1) mm = v[c] - v[c - 1];
-        val = fma(0.5, mm, v[c]);
+        const double d = sel == T + 2 ? 0.0 : (sel == T ? v[c + 1] : v[c - 1]) - v[c];
+        val = fma(sel == T + 1 ? -0.5 : 0.5, d, v[c]);
     }
     return val;
 }
