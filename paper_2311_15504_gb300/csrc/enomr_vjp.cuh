@@ -161,22 +161,6 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
     const double ph2_b = (C == 4) ? Fb[2] + FbE * vh : 0.0;
     const double ph0_b = acc_s_b - acc_d_b, pha_b = acc_s_b + acc_d_b;
 
-    // Component sums of the window with the weights of the full stencil on both
-    // sides.  A field with that choice (nearly all in smooth flow) has its sums
-    // over the window, and its part of the cells' cotangents, in common with the
-    // others up to factors of the field: X and Y once instead of eight sums per
-    // field, and one gather of G (below) instead of one per field.  A field on
-    // another choice takes no part in it and goes through the per-field path
-    // whole, so that no cell outside its stencils enters.  Both parts are left
-    // out where nothing needs them: the sums by warps, the gathers by CTAs.
-    // (FP64 pipe bound.  One transposed product, order 9, 512^2: smooth periodic
-    // flow 1.95 -> 1.36 ms with the common part; four-quadrant Riemann state,
-    // hardly any full stencil, 1.91 / 1.98 ms.)
-    double X[C], Y[C], GU[C], GF[C];
-    bool have = false;  // X and Y are set
-#pragma unroll
-    for (int q = 0; q < C; ++q) X[q] = Y[q] = GU[q] = GF[q] = 0.0;
-
     double ftv[C];
     double hq_b = 0.0, uh_b = 0.0, vh_b = 0.0, kap_b = 0.0, c2g_b = 0.0;
     double ab[3] = {0.0, 0.0, 0.0};
@@ -187,32 +171,71 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
 #pragma unroll
         for (int q = 0; q < C; ++q) cUb[c][q] = cFb[c][q] = 0.0;
 
-#pragma unroll 1
-    for (int f = 0; f < C; ++f) {
-        const bool shear = (C == 4 && f == 2);
-        double l0c, l1c, alpha;
-        int aidx;
-        if (shear) {
+    // scaled left-eigenvector row of field f and its split speed
+    auto row = [&](int f, double &l0c, double &l1c, double &alpha) {
+        if (C == 4 && f == 2) {
             l0c = -vh;
             l1c = 0.0;
             alpha = a_0;
-            aidx = 1;
         } else if (f == 0) {
             l0c = fma(uh, kap, hq);
             l1c = -(uh + kap);
             alpha = a_m;
-            aidx = 0;
         } else if (f == C - 1) {
             l0c = fma(-uh, kap, hq);
             l1c = -(uh - kap);
             alpha = a_p;
-            aidx = 2;
         } else {
             l0c = hq - c2g;
             l1c = -uh;
             alpha = a_0;
-            aidx = 1;
         }
+    };
+    // cotangent of field f's f^+ + f^-
+    auto field_bar = [&](int f) {
+        if (f == 0) return 0.25 * b1 * ph0_b;
+        if (f == C - 1) return 0.25 * b1 * pha_b;
+        if (C == 4 && f == 2) return 0.5 * ph2_b;
+        return -0.5 * b1 * ph1_b;
+    };
+    // Reverse of split and projection, per window cell.  With P, M the weights of
+    // the two sides times ftb and d = P - M, the cotangents are w_bar = alpha d
+    // and q_bar = P + M; the sums S[q] = sum_j d_j U_j[q] give both the U part of
+    // the row-coefficient cotangents (alpha S) and the alpha cotangent
+    // sum_j d_j w_j = l . S.  Here: row coefficients -> Roe scalars, alpha.
+    auto rows_bar = [&](int f, double l0c, double l1c, double alpha, double S0, double S1, double ST,
+                        double SE, double Q0, double Q1, double QT) {
+        const double l0b = fma(alpha, S0, Q0);
+        if (C == 4 && f == 2) {
+            ab[1] += fma(l0c, S0, ST);
+            vh_b -= l0b;
+            return;
+        }
+        const double l1b = fma(alpha, S1, Q1), ltb = C == 4 ? fma(alpha, ST, QT) : 0.0;
+        double a = fma(l0c, S0, SE);
+        a = fma(l1c, S1, a);
+        if (C == 4) a = fma(-vh, ST, a);
+        ab[f == 0 ? 0 : (f == C - 1 ? 2 : 1)] += a;
+        hq_b += l0b;
+        vh_b -= ltb;
+        if (f == 0) {
+            uh_b += l0b * kap - l1b;
+            kap_b += l0b * uh - l1b;
+        } else if (f == C - 1) {
+            uh_b -= l0b * kap + l1b;
+            kap_b += l1b - l0b * uh;
+        } else {
+            c2g_b -= l0b;
+            uh_b -= l1b;
+        }
+    };
+    unsigned common = 0;  // fields that the common part below takes
+
+#pragma unroll 1
+    for (int f = 0; f < C; ++f) {
+        const bool shear = (C == 4 && f == 2);
+        double l0c, l1c, alpha;
+        row(f, l0c, l1c, alpha);
         auto project_w = [&](int s) {
             if (shear) return fma(l0c, sU[0][line][s], sU[2][line][s]);
             double w = sU[C - 1][line][s];
@@ -248,141 +271,53 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
             const double fm = mr_value<R>(vm, sA, valid, selm);
             ftv[f] = fp + fm;
         }
-        // cotangent of this field's f^+ + f^-
-        double ftb;
-        if (f == 0) ftb = 0.25 * b1 * ph0_b;
-        else if (f == C - 1) ftb = 0.25 * b1 * pha_b;
-        else if (shear) ftb = 0.5 * ph2_b;
-        else ftb = -0.5 * b1 * ph1_b;
-        // reverse of split and projection, per window cell.  With P, M the
-        // weights of the two sides times ftb and d = P - M, the cotangents are
-        // w_bar = alpha d and q_bar = P + M; the sums S[q] = sum_j d_j U_j[q]
-        // give both the U part of the row-coefficient cotangents (alpha S) and
-        // the alpha cotangent sum_j d_j w_j = l . S.
-        const bool full = (selp | selm) == 0;
-        const bool other = owned && !full;
-        if (!have && __any_sync(FULL, owned && full)) {
-            have = true;
-#pragma unroll
-            for (int q = 0; q < C; ++q)
-#pragma unroll
-                for (int j = 0; j < 2 * g; ++j) {
-                    X[q] = fma(Coef<R>::m()[j], sU[q][line][p + j], X[q]);
-                    Y[q] = fma(Coef<R>::p()[j], sF[q][line][p + j], Y[q]);
-                }
+        if (!__syncthreads_or(owned && (selp | selm) != 0)) {
+            common |= 1u << f;
+            continue;
         }
+        const double ftb = field_bar(f);
+        // reconstruction weights of the frozen choice, times ftb
+        constexpr int c0 = g - 1;
+        double wp[W], wm[W];
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            wp[j] = (selp < T) ? sA[selp * W + j] * ftb : 0.0;
+            wm[j] = (selm < T) ? sA[selm * W + j] * ftb : 0.0;
+        }
+        if (selp == T) { wp[c0] = 0.5 * ftb; wp[c0 + 1] = 0.5 * ftb; }
+        if (selp == T + 1) { wp[c0] = 1.5 * ftb; wp[c0 - 1] = -0.5 * ftb; }
+        if (selp == T + 2) wp[c0] = ftb;
+        if (selm == T) { wm[c0] = 0.5 * ftb; wm[c0 + 1] = 0.5 * ftb; }
+        if (selm == T + 1) { wm[c0] = 1.5 * ftb; wm[c0 - 1] = -0.5 * ftb; }
+        if (selm == T + 2) wm[c0] = ftb;
         double S0 = 0.0, S1 = 0.0, ST = 0.0, SE = 0.0, Q0 = 0.0, Q1 = 0.0, QT = 0.0;
-        if (owned && full) {
-            S0 = ftb * X[0];
-            S1 = ftb * X[1];
-            SE = ftb * X[C - 1];
-            Q0 = ftb * Y[0];
-            Q1 = ftb * Y[1];
-            if (C == 4) {
-                ST = ftb * X[2 % C];
-                QT = ftb * Y[2 % C];
-            }
-            const double fa = ftb * alpha;
-            GU[0] = fma(fa, l0c, GU[0]);
-            GF[0] = fma(ftb, l0c, GF[0]);
-            if (shear) {
-                GU[2 % C] += fa;
-                GF[2 % C] += ftb;
-            } else {
-                GU[1] = fma(fa, l1c, GU[1]);
-                GF[1] = fma(ftb, l1c, GF[1]);
-                GU[C - 1] += fa;
-                GF[C - 1] += ftb;
-                if (C == 4) {
-                    GU[2 % C] = fma(-vh, fa, GU[2 % C]);
-                    GF[2 % C] = fma(-vh, ftb, GF[2 % C]);
-                }
-            }
-        }
-        const bool others = __syncthreads_or(other) != 0;
-        if (others) {
-            // the frozen choice's weights, times ftb
-            constexpr int c0 = g - 1;
-            double wp[W], wm[W];
 #pragma unroll
-            for (int j = 0; j < W; ++j) {
-                double a = (selp < T) ? sA[selp * W + j] : 0.0, b = (selm < T) ? sA[selm * W + j] : 0.0;
-                if (j == c0) {
-                    a = selp == T ? 0.5 : (selp == T + 1 ? 1.5 : (selp == T + 2 ? 1.0 : a));
-                    b = selm == T ? 0.5 : (selm == T + 1 ? 1.5 : (selm == T + 2 ? 1.0 : b));
-                }
-                if (j == c0 + 1) {
-                    a = selp == T ? 0.5 : a;
-                    b = selm == T ? 0.5 : b;
-                }
-                if (j == c0 - 1) {
-                    a = selp == T + 1 ? -0.5 : a;
-                    b = selm == T + 1 ? -0.5 : b;
-                }
-                wp[j] = other ? a * ftb : 0.0;
-                wm[j] = other ? b * ftb : 0.0;
-            }
-#pragma unroll
-            for (int j = 0; j < 2 * g; ++j) {
-                const int s = p + j;
-                const double P = (j <= 2 * g - 2) ? wp[j] : 0.0;
-                const double M = (j >= 1) ? wm[2 * g - 1 - j] : 0.0;
-                const double qb = P + M, d = P - M;
-                sW.w.d[line][p][j] = d;  // alpha is folded into the gather's row
-                sW.w.q[line][p][j] = qb;
-                S0 = fma(d, sU[0][line][s], S0);
-                Q0 = fma(qb, sF[0][line][s], Q0);
-                if (C == 4) ST = fma(d, sU[2][line][s], ST);
-                if (!shear) {
-                    S1 = fma(d, sU[1][line][s], S1);
-                    SE = fma(d, sU[C - 1][line][s], SE);
-                    Q1 = fma(qb, sF[1][line][s], Q1);
-                    if (C == 4) QT = fma(qb, sF[2][line][s], QT);
-                }
+        for (int j = 0; j < 2 * g; ++j) {
+            const int s = p + j;
+            const double P = (j <= 2 * g - 2) ? wp[j] : 0.0;
+            const double M = (j >= 1) ? wm[2 * g - 1 - j] : 0.0;
+            const double qb = P + M, d = P - M;
+            sW.w.d[line][p][j] = d;  // alpha is folded into the gather's row
+            sW.w.q[line][p][j] = qb;
+            S0 = fma(d, sU[0][line][s], S0);
+            Q0 = fma(qb, sF[0][line][s], Q0);
+            if (C == 4) ST = fma(d, sU[2][line][s], ST);
+            if (!shear) {
+                S1 = fma(d, sU[1][line][s], S1);
+                SE = fma(d, sU[C - 1][line][s], SE);
+                Q1 = fma(qb, sF[1][line][s], Q1);
+                if (C == 4) QT = fma(qb, sF[2][line][s], QT);
             }
         }
-        double l0b, l1b = 0.0, ltb = 0.0;
-        l0b = fma(alpha, S0, Q0);
-        if (shear) {
-            ab[aidx] += fma(l0c, S0, ST);
-        } else {
-            l1b = fma(alpha, S1, Q1);
-            if (C == 4) ltb = fma(alpha, ST, QT);
-            double a = fma(l0c, S0, SE);
-            a = fma(l1c, S1, a);
-            if (C == 4) a = fma(-vh, ST, a);
-            ab[aidx] += a;
-        }
+        rows_bar(f, l0c, l1c, alpha, S0, S1, ST, SE, Q0, Q1, QT);
         // gather rows: U part scaled by alpha (it multiplies d), F part not
-        if (others) {
-            sRow[line][p][0] = l0c;
-            sRow[line][p][1] = l1c;
-            sRow[line][p][2] = (C == 4) ? -vh : 0.0;
-            sRowA[line][p][0] = alpha * l0c;
-            sRowA[line][p][1] = alpha * l1c;
-            sRowA[line][p][2] = (C == 4) ? -alpha * vh : 0.0;
-            sRowA[line][p][3] = alpha;
-        }
-        // row coefficients -> Roe scalars
-        if (shear) {
-            vh_b -= l0b;
-        } else if (f == 0) {
-            hq_b += l0b;
-            uh_b += l0b * kap - l1b;
-            kap_b += l0b * uh - l1b;
-            vh_b -= ltb;
-        } else if (f == C - 1) {
-            hq_b += l0b;
-            uh_b -= l0b * kap + l1b;
-            kap_b += l1b - l0b * uh;
-            vh_b -= ltb;
-        } else {
-            hq_b += l0b;
-            c2g_b -= l0b;
-            uh_b -= l1b;
-            vh_b -= ltb;
-        }
-        if (!others) continue;
+        sRow[line][p][0] = l0c;
+        sRow[line][p][1] = l1c;
+        sRow[line][p][2] = (C == 4) ? -vh : 0.0;
+        sRowA[line][p][0] = alpha * l0c;
+        sRowA[line][p][1] = alpha * l1c;
+        sRowA[line][p][2] = (C == 4) ? -alpha * vh : 0.0;
+        sRowA[line][p][3] = alpha;
         __syncthreads();
         // gather: staged cell s receives wb l and qb l from interfaces p' = s - j
 #pragma unroll
@@ -428,34 +363,82 @@ __global__ void __launch_bounds__(TP *NL) k_sweep_vjp(VjpArgs A)
         __syncthreads();
     }
 
-    // ---- the common part of the fields: cell s receives the full stencil's
-    // weight of its place in the window of interface p' = s - j times G
+    // ---- Fields of which every interface of the CTA is on the full stencil on
+    // both sides (nearly all in smooth flow).  Their sums over the window, and
+    // their part of the cells' cotangents, are common up to factors of the field:
+    // X and Y once instead of eight sums per field, and one gather of G instead of
+    // one per field.  The others went through the loop above whole, their full
+    // stencils included, so that no cell outside the chosen stencils enters and
+    // nothing is done twice; and this part's sums are not alive in the loop, whose
+    // registers set the occupancy (order 5: 166 registers, six CTAs per SM, 190
+    // and five with them).  FP64 pipe bound.  One transposed product, 1024^2, every
+    // field by itself / this: smooth periodic flow, order 5, 5.21 / 4.03 ms, order
+    // 9, 7.62 / 5.79, order 17, 13.6 / 10.8; quadrants of constant states, hardly
+    // any full stencil, 4.65 / 4.78, 6.48 / 6.65, 10.1 / 10.4.
+    if (common) {
+        double X[C], Y[C], GU[C], GF[C];
 #pragma unroll
-    for (int q = 0; q < C; ++q) {
-        sW.G[line][p][q] = GU[q];
-        sW.G[line][p][C + q] = GF[q];
-    }
-    const bool common = __syncthreads_or(have) != 0;
-#pragma unroll
-    for (int c = 0; c < CPT && common; ++c) {
-        const int idx = tid + c * NT;
-        if (idx < NL * S) {
-            int gl, s;
-            if (DIR == 0) {
-                gl = idx / S;
-                s = idx - gl * S;
-            } else {
-                s = idx / NL;
-                gl = idx - s * NL;
-            }
+        for (int q = 0; q < C; ++q) {
+            X[q] = Y[q] = GU[q] = GF[q] = 0.0;
 #pragma unroll
             for (int j = 0; j < 2 * g; ++j) {
-                const int pp = s - j;
-                if (pp < 0 || pp >= TP) continue;
+                X[q] = fma(Coef<R>::m()[j], sU[q][line][p + j], X[q]);
+                Y[q] = fma(Coef<R>::p()[j], sF[q][line][p + j], Y[q]);
+            }
+        }
 #pragma unroll
-                for (int q = 0; q < C; ++q) {
-                    cUb[c][q] = fma(Coef<R>::m()[j], sW.G[gl][pp][q], cUb[c][q]);
-                    cFb[c][q] = fma(Coef<R>::p()[j], sW.G[gl][pp][C + q], cFb[c][q]);
+        for (int f = 0; f < C; ++f) {
+            if (!(common & (1u << f)) || !owned) continue;
+            double l0c, l1c, alpha;
+            row(f, l0c, l1c, alpha);
+            const double ftb = field_bar(f), fa = ftb * alpha;
+            rows_bar(f, l0c, l1c, alpha, ftb * X[0], ftb * X[1], C == 4 ? ftb * X[2 % C] : 0.0,
+                     ftb * X[C - 1], ftb * Y[0], ftb * Y[1], C == 4 ? ftb * Y[2 % C] : 0.0);
+            GU[0] = fma(fa, l0c, GU[0]);
+            GF[0] = fma(ftb, l0c, GF[0]);
+            if (C == 4 && f == 2) {
+                GU[2 % C] += fa;
+                GF[2 % C] += ftb;
+            } else {
+                GU[1] = fma(fa, l1c, GU[1]);
+                GF[1] = fma(ftb, l1c, GF[1]);
+                GU[C - 1] += fa;
+                GF[C - 1] += ftb;
+                if (C == 4) {
+                    GU[2 % C] = fma(-vh, fa, GU[2 % C]);
+                    GF[2 % C] = fma(-vh, ftb, GF[2 % C]);
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < C; ++q) {
+            sW.G[line][p][q] = GU[q];
+            sW.G[line][p][C + q] = GF[q];
+        }
+        __syncthreads();
+        // cell s receives the full stencil's weight of its place in the window of
+        // interface p' = s - j times G
+#pragma unroll
+        for (int c = 0; c < CPT; ++c) {
+            const int idx = tid + c * NT;
+            if (idx < NL * S) {
+                int gl, s;
+                if (DIR == 0) {
+                    gl = idx / S;
+                    s = idx - gl * S;
+                } else {
+                    s = idx / NL;
+                    gl = idx - s * NL;
+                }
+#pragma unroll
+                for (int j = 0; j < 2 * g; ++j) {
+                    const int pp = s - j;
+                    if (pp < 0 || pp >= TP) continue;
+#pragma unroll
+                    for (int q = 0; q < C; ++q) {
+                        cUb[c][q] = fma(Coef<R>::m()[j], sW.G[gl][pp][q], cUb[c][q]);
+                        cFb[c][q] = fma(Coef<R>::p()[j], sW.G[gl][pp][C + q], cFb[c][q]);
+                    }
                 }
             }
         }
