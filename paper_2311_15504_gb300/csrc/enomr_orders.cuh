@@ -17,14 +17,20 @@ constexpr int ADV_TP = 256;
 template <int R> cudaError_t launch_advection(const AdvArgs &a, cudaStream_t s)
 {
     const long long tiles = (a.n + ADV_TP - 2) / (ADV_TP - 1);
-    k_advection<R, ADV_TP><<<(unsigned)tiles, ADV_TP, 0, s>>>(a);
+    if (tiles <= SCALAR_FEW_TILES)
+        k_advection<R, ADV_TP, 1><<<(unsigned)tiles, ADV_TP, 0, s>>>(a);
+    else
+        k_advection<R, ADV_TP, SCALAR_CTAS><<<(unsigned)tiles, ADV_TP, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 template <int R> cudaError_t launch_burgers(const AdvArgs &a, cudaStream_t s)
 {
     const long long tiles = (a.n + ADV_TP - 2) / (ADV_TP - 1);
-    k_burgers<R, ADV_TP><<<(unsigned)tiles, ADV_TP, 0, s>>>(a);
+    if (tiles <= SCALAR_FEW_TILES)
+        k_burgers<R, ADV_TP, 1><<<(unsigned)tiles, ADV_TP, 0, s>>>(a);
+    else
+        k_burgers<R, ADV_TP, SCALAR_CTAS><<<(unsigned)tiles, ADV_TP, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -75,27 +75,34 @@ __device__ __forceinline__ double scalar_value(const double *v0, const float2 *e
     return value;
 }
 
+// From global memory: a warp reads constant memory one address at a time (order
+// 17, 416 entries: 2e6 cells, one right-hand side 83 -> 55 us; 300 000 cells with a
+// square pulse 22.6 -> 17.2 us).
 template <int R>
 __device__ __forceinline__ void load_w_table(float2 *sW, int tid, int nthreads)
 {
     constexpr int N = R - 1;
-    for (int i = tid; i < Tab<R>::T * N; i += nthreads) sW[i] = Coef<R>::w()[i];
+    for (int i = tid; i < Tab<R>::T * N; i += nthreads) sW[i] = Coef<R>::w_table()[i];
 }
 
-// Resident CTAs (of 256 threads) per SM of the scalar kernels, 32 registers:
-// between the FP64 operations lie long float sums, and more warps fill the
-// FP64 pipe's gaps although the sums spill.  Burgers, N = 2^22, order 9 / 13 /
-// 17: 123 / 167 / 277 us a launch unbounded (58 to 84 registers), 117 / 141 /
-// 196 with five, 114 / 127 / 181 with eight; advection, N = 1 048 573, order 17:
-// 65 -> 52.
+// Resident CTAs (of 256 threads) per SM of the scalar kernels.  Long lines,
+// eight of 32 registers: between the FP64 operations lie long float sums, and
+// more warps fill the FP64 pipe's gaps although the sums spill.  Burgers, N =
+// 2^22, order 9 / 13 / 17: 123 / 167 / 277 us a launch unbounded (58 to 84
+// registers), 117 / 141 / 196 with five, 114 / 127 / 181 with eight; advection,
+// N = 1 048 573, order 17: 65 -> 52.  Lines of at most two CTAs per SM, whose
+// launches last as long as one CTA: unbounded, without the spills (Burgers, order
+// 17, 3000 cells, five stages of the linear SSP family: 90 -> 79 us; 300 000 cells,
+// 1177 CTAs: 137 with eight, 157 unbounded).
 constexpr int SCALAR_CTAS = 8;
+constexpr long long SCALAR_FEW_TILES = 2 * 152;
 
 // ---------------------------------------------------------------------------
 // Scalar advection f(u) = a u, alpha = |a|: f^+ = a u, f^- = 0 for a >= 0
 // (mirror for a < 0).  One thread per interface.
 // ---------------------------------------------------------------------------
-template <int R, int TP>
-__global__ void __launch_bounds__(TP, SCALAR_CTAS) k_advection(AdvArgs A)
+template <int R, int TP, int MINB>
+__global__ void __launch_bounds__(TP, MINB) k_advection(AdvArgs A)
 {
     constexpr int g = (R + 1) / 2, W = 2 * g - 1, S = TP + 2 * g - 1, T = Tab<R>::T;
     __shared__ double sf[S];
@@ -143,8 +150,8 @@ __global__ void __launch_bounds__(TP, SCALAR_CTAS) k_advection(AdvArgs A)
 // the same state), so a warp never diverges on it.  One thread per
 // interface; split values are formed as written, 1/2 (f +- alpha u).
 // ---------------------------------------------------------------------------
-template <int R, int TP>
-__global__ void __launch_bounds__(TP, SCALAR_CTAS) k_burgers(AdvArgs A)
+template <int R, int TP, int MINB>
+__global__ void __launch_bounds__(TP, MINB) k_burgers(AdvArgs A)
 {
     constexpr int g = (R + 1) / 2, W = 2 * g - 1, S = TP + 2 * g - 1, T = Tab<R>::T;
     __shared__ double sp[S];

@@ -177,10 +177,13 @@ def generate() -> str:
                        + ", ".join(hexlit(full[j] + sg * full[2 * g - 1 - j]) for j in range(2 * g)) + "};")
         out.append("// {high, rest} of the difference weights w_j of every row")
         for name, rows in ((f"kW{R}", [difference_weights(r, g - 1) for r in as_]),):
-            out.append(f"static __constant__ float2 {name}[{sum(len(r) for r in rows)}] = {{")
-            for row in rows:
-                out.append("    " + ", ".join("{%s, %s}" % tuple(map(flit, pair(x))) for x in row) + ",")
-            out.append("};")
+            # the full stencil's as constant operands; all rows in global memory:
+            # a warp reads constant memory one address at a time
+            for kind, nm, rs in (("__constant__", name, rows[:1]), ("__device__ const", name + "T", rows)):
+                out.append(f"static {kind} float2 {nm}[{sum(len(r) for r in rs)}] = {{")
+                for row in rs:
+                    out.append("    " + ", ".join("{%s, %s}" % tuple(map(flit, pair(x))) for x in row) + ",")
+                out.append("};")
         out.append("")
     out.append("template <int R> struct Coef;")
     for R in ORDERS:
@@ -194,6 +197,7 @@ def generate() -> str:
             out.append(f"    __device__ static __forceinline__ const double *{f.lower()}() {{ return k{f}{R}; }}")
         for f in "W":
             out.append(f"    __device__ static __forceinline__ const float2 *{f.lower()}() {{ return k{f}{R}; }}")
+            out.append(f"    __device__ static __forceinline__ const float2 *{f.lower()}_table() {{ return k{f}{R}T; }}")
         out.append("};")
     out.append("")
     out.append("}  // namespace enomr")
