@@ -33,7 +33,14 @@ __device__ __forceinline__ double scalar_value(const double *v0, const float2 *e
     const float vc = fabsf(to_float(v0[DIRN * c]));
     const bool left0 = e[c - 1] == 0.0f && e[c - 2] == 0.0f;
     const bool right0 = e[c] == 0.0f && e[c + 1] == 0.0f;
-    sel = select_float<R>(e, vc, left0, right0);
+    // a warp of which every window is constant up to rounding or exactly: mr_select
+    const bool none = left0 || right0;
+    const float near = fmaxf(fmaxf(fabsf(e[c - 2]), fabsf(e[c - 1])), fmaxf(fabsf(e[c]), fabsf(e[c + 1])));
+    const bool noise = !none && near <= vc * (0x1p-52f * (float)NOISE_ULP<R>);
+    if (__all_sync(FULL, noise || none || !valid))
+        sel = none ? T + 2 : SEL_OPEN;
+    else
+        sel = select_float<R>(e, vc, left0, right0);
     const bool open = valid && sel == SEL_OPEN;
     if (__any_sync(FULL, open)) {
         double v[W];
@@ -43,15 +50,20 @@ __device__ __forceinline__ double scalar_value(const double *v0, const float2 *e
         mr_select64<R>(v, open, s64);
         if (open) sel = s64;
     }
-    // NaN differences do not enter emax: the float selection was open then
-    bool small = emax <= PAIR_RANGE * vc && sel < T && valid;
+    // NaN differences do not enter emax: the float selection was open then.  An
+    // open window has spent its FP64 time already and takes the FP64 sum; so does
+    // one that may have been left open for the sake of its warp.
+    bool small = emax <= PAIR_RANGE * vc && sel < T && valid && !open && !noise;
 #pragma unroll
     for (int j = 0; j < N; ++j) small = small && e[j] == e[j];
     // the form is each lane's own choice: the face shared by two tiles takes
     // the same one in both
     auto rest = [&](int j) { return DIRN > 0 ? e0[j] : make_float2(-e0[-j].x, -e0[-j].y); };
     double value = 0.0;
-    if (__all_sync(FULL, !small || sel == 0)) {
+    const unsigned pairs = __ballot_sync(FULL, small);
+    if (pairs == 0) {
+        // none
+    } else if (__all_sync(FULL, !small || sel == 0)) {
         PairSum q;
         q.first(Coef<R>::w()[0], rest(0));
 #pragma unroll
