@@ -534,18 +534,16 @@ __global__ void __launch_bounds__(256) k_scalar_speed(const double *U, long long
         m = m > a ? m : a;
         if (a != 0) fl |= (b < 0) ? SGN_NEG : SGN_POS;
     };
-    // eight loads in flight per thread: the launch is bound by the latency of
-    // its reads otherwise (N = 2^22: 21 us with one)
+    // eight loads in flight per thread, the last ones of a line too: the launch
+    // is bound by the latency of its reads otherwise (N = 2^22: 21 us with one)
     const long long stride = (long long)gridDim.x * blockDim.x;
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; i + 7 * stride < n; i += 8 * stride) {
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += 8 * stride) {
         double u[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) u[j] = U[i + j * stride];
+        for (int j = 0; j < 8; ++j) u[j] = i + j * stride < n ? U[i + j * stride] : 0.0;
 #pragma unroll
         for (int j = 0; j < 8; ++j) take(u[j]);
     }
-    for (; i < n; i += stride) take(U[i]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long w = __shfl_xor_sync(0xffffffffu, m, o);
