@@ -117,7 +117,7 @@ struct AdvArgs {
 };
 
 // One SSP-RK3 step of a scalar line of at most SMALL_CELLS cells (enomr_scalar.cuh)
-constexpr int SMALL_CELLS = 1024, SMALL_THREADS = 512;
+constexpr int SMALL_CELLS = 1024, SMALL_TILE = 255, SMALL_THREADS = 256;  // tile: cells per CTA
 struct SmallArgs {
     double *U;             // [n], in place
     long long n;

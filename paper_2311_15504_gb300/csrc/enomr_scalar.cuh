@@ -3,6 +3,8 @@
 // One thread per interface; a CTA stages TP + 2g - 1 split flux values.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include "enomr_select.cuh"
 
 namespace enomr {
@@ -264,21 +266,27 @@ __global__ void __launch_bounds__(TP, MINB) k_burgers(AdvArgs A)
 namespace enomr {
 
 // ---------------------------------------------------------------------------
-// One SSP-RK3 step of a short scalar line in one launch of one CTA: the state,
-// its fluxes and their differences stay in shared memory through the three
-// stages, with the same operations per cell and interface as k_advection and
-// k_burgers.  A line of n <= SMALL_CELLS is a few warps of work; launched one
-// stage at a time it costs four (Burgers: seven) launches of about 5 us each.
-// Measured per step (advection, order 5, n = 200, ten steps in a row): 20.7 ->
-// 11.9 us.  Up to SMALL_CELLS = 1024 cells: there the one SM's FP64 work (about
-// 12 operations a cell and stage) is still below a launch.
+// One SSP-RK3 step of a short scalar line in one launch: a cluster of CTAs, each
+// with up to SMALL_TILE cells, their interfaces one per thread.  Every CTA holds
+// the state of the whole line in shared memory; a stage's new cells go to all of
+// them (distributed shared memory), one cluster barrier a stage.  The same
+// operations per cell and interface as k_advection and k_burgers, and as many
+// cells on an SM, so that the FP64 work of windows that the float form leaves
+// open is spread as in their launches.  A line of n <= SMALL_CELLS is a few warps
+// of work; launched one stage at a time it costs four (Burgers: seven) launches
+// of about 5 us each.  A step, by launches of one stage each / in one CTA / over a
+// cluster: advection, order 5, 200 cells 23.7 / 15.7 / 15.8 us; 1024 cells, smooth
+// 23.8 / 21.5 / 14.1, constant up to rounding 27 / 58 / 20; order 17, random cells
+// 92 / 56 / 20, constant up to rounding 92 / 325 / 77; Burgers, order 9, smooth
+// 43 / 25 / 16.
 // ---------------------------------------------------------------------------
 template <int R, bool BURGERS>
 struct SmallSmem {
-    static constexpr int g = (R + 1) / 2, W = 2 * g - 1, T = Tab<R>::T, N = SMALL_CELLS;
-    double u0[N], u[N], fh[N + 1];
-    double f[BURGERS ? 2 : 1][N + 2 * g];   // f^+ (advection: the flux), f^-
-    float2 e[BURGERS ? 2 : 1][N + 2 * g];
+    static constexpr int g = (R + 1) / 2, W = 2 * g - 1, T = Tab<R>::T, S = SMALL_TILE + 2 * g;
+    double u[2][SMALL_CELLS];               // the stage's state, the next one's
+    double fh[SMALL_TILE + 1];
+    double f[BURGERS ? 2 : 1][S];           // f^+ (advection: the flux), f^-
+    float2 e[BURGERS ? 2 : 1][S];
     double a[T * W];
     float2 w[T * (W - 1)];
     double dt, alpha;
@@ -290,83 +298,90 @@ template <int R, bool BURGERS>
 __global__ void __launch_bounds__(SMALL_THREADS) k_scalar_step(SmallArgs A)
 {
     constexpr int g = (R + 1) / 2, T = Tab<R>::T;
-    extern __shared__ __align__(16) unsigned char smem_small[];
     using SM = SmallSmem<R, BURGERS>;
-    SM &sm = *reinterpret_cast<SM *>(smem_small);
+    __shared__ SM sm;
+    auto cluster = cooperative_groups::this_cluster();
     const int tid = threadIdx.x, n = (int)A.n;
+    const int ctas = (int)gridDim.x, rank = (int)blockIdx.x;  // one cluster
+    const int chunk = (n + ctas - 1) / ctas, c0 = rank * chunk;
+    const int m = chunk < n - c0 ? chunk : n - c0;            // this CTA's cells: c0 ..
     load_a_table<R>(sm.a, tid, SMALL_THREADS);
     load_w_table<R>(sm.w, tid, SMALL_THREADS);
-    for (int i = tid; i < n; i += SMALL_THREADS) sm.u0[i] = sm.u[i] = A.U[i];
+    for (int i = tid; i < n; i += SMALL_THREADS) sm.u[0][i] = A.U[i];
     if (tid == 0) {
         sm.dt = A.dt_fixed;
         sm.mode = A.a >= 0.0 ? 0 : 1;  // advection: the upwind side
     }
-    __syncthreads();
+    // the line is read by all and every CTA has started: it may be written
+    cluster.sync();
+    const double u0 = tid < m ? sm.u[0][c0 + tid] : 0.0;
     for (int stage = 0; stage < 3; ++stage) {
+        const double *u = sm.u[stage & 1];
         if constexpr (BURGERS) {
             // k_scalar_speed: max |u|, and which signs occur
-            unsigned long long m = 0, fl = 0;
+            unsigned long long mx = 0, fl = 0;
             for (int i = tid; i < n; i += SMALL_THREADS) {
-                const long long b = __double_as_longlong(sm.u[i]);
+                const long long b = __double_as_longlong(u[i]);
                 const unsigned long long x = (unsigned long long)(b & 0x7fffffffffffffffLL);
-                if (!below_1e300(sm.u[i])) atomicOr(A.status, ST_NONPHYS_CELL);
-                m = m > x ? m : x;
+                if (!below_1e300(u[i])) atomicOr(A.status, ST_NONPHYS_CELL);
+                mx = mx > x ? mx : x;
                 if (x != 0) fl |= (b < 0) ? SGN_NEG : SGN_POS;
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
-                const unsigned long long x = __shfl_xor_sync(FULL, m, o);
-                m = m > x ? m : x;
+                const unsigned long long x = __shfl_xor_sync(FULL, mx, o);
+                mx = mx > x ? mx : x;
                 fl |= __shfl_xor_sync(FULL, fl, o);
             }
             if ((tid & 31) == 0) {
-                sm.red[tid >> 5][0] = m;
+                sm.red[tid >> 5][0] = mx;
                 sm.red[tid >> 5][1] = fl;
             }
             __syncthreads();
             if (tid == 0) {
                 for (int i = 1; i < SMALL_THREADS / 32; ++i) {
-                    m = m > sm.red[i][0] ? m : sm.red[i][0];
+                    mx = mx > sm.red[i][0] ? mx : sm.red[i][0];
                     fl |= sm.red[i][1];
                 }
-                sm.alpha = __longlong_as_double((long long)m);
+                sm.alpha = __longlong_as_double((long long)mx);
                 sm.mode = !(fl & SGN_NEG) ? 0 : (!(fl & SGN_POS) ? 1 : 2);
                 if (stage == 0)
                     sm.dt = step_size(__dmul_rn(sm.alpha, A.inv_h), A.cfl, A.dt_fixed);
-                A.speed[0] = sm.alpha;
-                A.speed[1] = __longlong_as_double((long long)fl);
+                if (rank == 0) {
+                    A.speed[0] = sm.alpha;
+                    A.speed[1] = __longlong_as_double((long long)fl);
+                }
             }
             __syncthreads();
         }
         const int mode = sm.mode;
         // split fluxes with their ghost cells, then their differences
-        for (int s = tid; s < n + 2 * g; s += SMALL_THREADS) {
-            const double u = sm.u[ghost(s - g, n, A.bc)];
+        for (int s = tid; s < m + 2 * g; s += SMALL_THREADS) {
+            const double us = u[ghost(c0 + s - g, n, A.bc)];
             if constexpr (BURGERS) {
-                const double f = 0.5 * __dmul_rn(u, u);
+                const double f = 0.5 * __dmul_rn(us, us);
                 double fp = f, fm = f;
                 if (mode == 2) {
-                    const double au = __dmul_rn(sm.alpha, u);
+                    const double au = __dmul_rn(sm.alpha, us);
                     fp = 0.5 * __dadd_rn(f, au);
                     fm = 0.5 * __dsub_rn(f, au);
                 }
                 sm.f[0][s] = fp;
                 sm.f[BURGERS ? 1 : 0][s] = fm;
             } else {
-                sm.f[0][s] = A.a * u;
+                sm.f[0][s] = A.a * us;
             }
         }
         __syncthreads();
-        for (int s = tid; s < n + 2 * g - 1; s += SMALL_THREADS) {
+        for (int s = tid; s < m + 2 * g - 1; s += SMALL_THREADS) {
             if (!BURGERS || mode != 1) sm.e[0][s] = split_pair(sm.f[0][s + 1] - sm.f[0][s]);
             if (BURGERS && mode != 0)
                 sm.e[BURGERS ? 1 : 0][s] = split_pair(sm.f[BURGERS ? 1 : 0][s + 1] - sm.f[BURGERS ? 1 : 0][s]);
         }
         __syncthreads();
-        for (int base = tid & ~31; base <= n; base += SMALL_THREADS) {
-            const int k = base + (tid & 31);  // interface x_{k-1/2}
-            const bool valid = k <= n;
-            const int p = valid ? k : n;
+        if ((tid & ~31) <= m) {  // interface x_{c0+tid-1/2}
+            const bool valid = tid <= m;
+            const int p = valid ? tid : m;
             int sel = T + 2;
             double hp = 0.0, hm = 0.0;
             if (mode != 1)
@@ -376,39 +391,43 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_scalar_step(SmallArgs A)
                 hm = scalar_value<R, -1>(sm.f[q] + p + 2 * g - 1, sm.e[q] + p + 2 * g - 2, sm.a, sm.w,
                                          valid, sel);
             }
-            if (valid) sm.fh[k] = BURGERS ? __dadd_rn(hp, hm) : (mode != 1 ? hp : hm);
+            if (valid) sm.fh[tid] = BURGERS ? __dadd_rn(hp, hm) : (mode != 1 ? hp : hm);
         }
         __syncthreads();
-        const double dt = sm.dt;
-        for (int i = tid; i < n; i += SMALL_THREADS) {
-            const double D = __dmul_rn(-(sm.fh[i + 1] - sm.fh[i]), A.inv_h);
-            const double w = fma(dt, D, sm.u[i]);
-            const double o = stage == 0 ? w : fma(A.c0[stage], sm.u0[i], A.c1[stage] * w);
-            sm.u[i] = o;
-            if (stage == 2) A.U[i] = o;
+        if (tid < m) {
+            const double D = __dmul_rn(-(sm.fh[tid + 1] - sm.fh[tid]), A.inv_h);
+            const double w = fma(sm.dt, D, u[c0 + tid]);
+            const double o = stage == 0 ? w : fma(A.c0[stage], u0, A.c1[stage] * w);
+            if (stage == 2) {
+                A.U[c0 + tid] = o;
+            } else {
+                double *next = &sm.u[(stage + 1) & 1][c0 + tid];
+                for (int r = 0; r < ctas; ++r) *cluster.map_shared_rank(next, r) = o;
+            }
         }
-        __syncthreads();
+        // every CTA has the next state, and none reads this one's any more; after
+        // the last stage nothing of another CTA is written
+        if (stage < 2) cluster.sync();
     }
-    if (tid == 0) *A.dt = sm.dt;
+    if (rank == 0 && tid == 0) *A.dt = sm.dt;
 }
 
 template <int R> cudaError_t launch_scalar_step(const SmallArgs &a, bool burgers, cudaStream_t s)
 {
-    const size_t bytes = burgers ? sizeof(SmallSmem<R, true>) : sizeof(SmallSmem<R, false>);
-    auto k = burgers ? k_scalar_step<R, true> : k_scalar_step<R, false>;
-    constexpr int kMaxDev = 64;
-    static bool granted[2][kMaxDev] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDev) return cudaErrorInvalidDevice;
-    if (!granted[burgers][dev]) {
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e != cudaSuccess) return e;
-        granted[burgers][dev] = true;
-    }
-    k<<<1, SMALL_THREADS, bytes, s>>>(a);
-    return cudaGetLastError();
+    static_assert(SMALL_CELLS <= 8 * SMALL_TILE, "a portable cluster");
+    static_assert(SMALL_THREADS > SMALL_TILE, "one interface per thread");
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)((a.n + SMALL_TILE - 1) / SMALL_TILE);
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(attr.val.clusterDim.x);
+    cfg.blockDim = dim3(SMALL_THREADS);
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return burgers ? cudaLaunchKernelEx(&cfg, k_scalar_step<R, true>, a)
+                   : cudaLaunchKernelEx(&cfg, k_scalar_step<R, false>, a);
 }
 
 }  // namespace enomr
