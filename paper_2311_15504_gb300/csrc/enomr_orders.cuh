@@ -104,16 +104,26 @@ template cudaError_t launch_euler2d_y_ext<ENOMR_R>(const SweepArgs &, bool, cuda
 
 namespace enomr {
 
+template <int R, int TP>
+cudaError_t launch_batch_tile(const BatchArgs &a, int grid, cudaStream_t s)
+{
+    const long long items = (a.ntiles + a.tiles_per_item - 1) / a.tiles_per_item;
+    if ((items < grid ? items : grid) * TP <= BATCH_FEW_THREADS_PER_SM * 152LL)
+        k_batch_stage<R, TP, BATCH_FEW_THREADS_PER_SM><<<grid, TP, 0, s>>>(a);
+    else
+        k_batch_stage<R, TP, BATCH_THREADS_PER_SM><<<grid, TP, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 template <int R> cudaError_t launch_batch_stage(const BatchArgs &a, int tp, int grid,
                                                 cudaStream_t s)
 {
     switch (tp) {
-    case 32: k_batch_stage<R, 32><<<grid, 32, 0, s>>>(a); break;
-    case 64: k_batch_stage<R, 64><<<grid, 64, 0, s>>>(a); break;
-    case 128: k_batch_stage<R, 128><<<grid, 128, 0, s>>>(a); break;
+    case 32: return launch_batch_tile<R, 32>(a, grid, s);
+    case 64: return launch_batch_tile<R, 64>(a, grid, s);
+    case 128: return launch_batch_tile<R, 128>(a, grid, s);
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 template cudaError_t launch_batch_stage<ENOMR_R>(const BatchArgs &, int, int, cudaStream_t);

@@ -1006,16 +1006,19 @@ __global__ void __launch_bounds__(TP *NL, MINB) k_sweep(SweepArgs A)
 // size.  Each tile runs the same interface arithmetic as the single-problem
 // sweep, so results are bitwise those of one problem at a time.
 // ---------------------------------------------------------------------------
-// Resident threads per SM: 1024 (64 registers).  Most tiles hold one state and
+// Resident threads per SM (THREADS): 1024 (64 registers).  Most tiles hold one state and
 // are a chain of loads and barriers, so the rate is set by how many are in
 // flight; left to itself the kernel takes 155 to 255 registers, 4 to 6 CTAs of
 // 64 threads.  4096 Riemann problems, a step at order 5 / 9 / 17: 2.15 / 2.83 /
 // 4.11 ms unbounded, 1.65 / 1.89 / 2.71 ms with 1024 threads, 2.03 / 2.22 / 2.98
 // with 768, 1.74 / 1.93 / 2.76 with 1280; twenty steps later 3.79 / 5.59 / 16.8
-// against 2.90 / 4.67 / 11.9 ms.
-constexpr int BATCH_THREADS_PER_SM = 1024;
-template <int R, int TP>
-__global__ void __launch_bounds__(TP, BATCH_THREADS_PER_SM / TP) k_batch_stage(BatchArgs B)
+// against 2.90 / 4.67 / 11.9 ms.  Batches whose CTAs fit on the chip with 256
+// threads per SM, where a launch lasts as long as one tile: 256, without spills
+// (order 17, 64 problems of 500 cells, smooth / constant up to rounding: 237 / 788
+// -> 189 / 614 us a step; one problem of 300 cells 163 / 472 -> 135 / 354).
+constexpr int BATCH_THREADS_PER_SM = 1024, BATCH_FEW_THREADS_PER_SM = 256;
+template <int R, int TP, int THREADS>
+__global__ void __launch_bounds__(TP, THREADS / TP) k_batch_stage(BatchArgs B)
 {
     constexpr int g = (R + 1) / 2, W = 2 * g - 1, T = Tab<R>::T;
     __shared__ SweepSmem<R, 3, TP, 1> sm;
