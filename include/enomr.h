@@ -266,11 +266,11 @@ ENOMR_API enomr_status enomr_set_staging(enomr_ctx *ctx, int mode);
  *                         long path's windows stay in registers): for grids
  *                         of few tiles, whose launches last as long as a
  *                         few tiles in sequence;
- *   ENOMR_OCCUPANCY_AUTO  (default) HIGH where the sweeps go by a list of
- *                         tiles (enomr_set_staging); over all tiles LOW when
- *                         the x sweep has fewer of them than four waves of
- *                         the HIGH instance (grids up to about 900^2), else
- *                         HIGH.
+ *   ENOMR_OCCUPANCY_AUTO  (default) LOW when the x sweep has fewer tiles
+ *                         than four waves of the HIGH instance (grids up to
+ *                         about 900^2), where the sweeps go by a list of
+ *                         tiles (enomr_set_staging) 7/4 waves (up to about
+ *                         500^2); else HIGH.
  * On smooth data the two are alike (1024^2 vortex: 6.67 / 6.73 ms a step); on
  * piecewise-constant data HIGH is faster (4096^2, order 9: 2.95 / 4.08 ms).
  * Same results bit for bit.  Host-only setting, no synchronisation.

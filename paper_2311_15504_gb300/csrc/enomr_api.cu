@@ -855,18 +855,23 @@ static SweepArgs sweep_args(enomr_ctx *c, const double *U, bool ysweep)
     return a;
 }
 
-// The 2D sweeps' low-occupancy instances: forced, or (automatic) over all
-// tiles of grids whose x sweep has fewer tiles than four waves of the
-// high-occupancy instance, whose launches last as long as a few tiles in
-// sequence.  Over a list the high-occupancy instance (Riemann states, a step:
-// 801^2 order 5 0.26 against 0.30 ms, 1024^2 order 9 0.96 / 1.02, 2048^2
-// order 13 2.33 / 2.81, order 17 3.66 / 4.42, 4096^2 order 9 3.01 / 4.18).
+// The 2D sweeps' low-occupancy instances: forced, or (automatic) on grids whose
+// x sweep has fewer tiles than four waves of the high-occupancy instance over all
+// tiles, 7/4 over a list: their launches last as long as a few tiles in sequence.
+// Over a list, Riemann states, a step with the low over the high instance at t = 0
+// / after 20 / 150 steps: 256 x 258 (384 tiles), order 5 0.97 / 0.90 / 0.82, order
+// 17 0.88 / 0.88 / 0.84; 512^2 (1280), order 5 0.98 / 0.83 / 1.0, order 9 0.96 /
+// 0.76 / 0.87, order 17 0.87 / 0.76 / 0.87; two sets of fronts (periodic) 1.2 /
+// 1.0 / 0.9.  300 x 1200 (1500), periodic: 1.3 / 1.0 / 0.96; 801^2 (2807), order 5
+// 1.08 / 0.83 / 0.96, order 9 1.06 / 0.82 / 0.92; 1024^2, order 9 1.09 / 0.95 /
+// 0.90; 2048^2, order 17 1.37 / 0.94; 4096^2, order 9, after 24 steps 1.38.
 static bool low_occupancy(const enomr_ctx *c, bool list)
 {
     if (c->occupancy == ENOMR_OCCUPANCY_LOW) return true;
-    if (c->occupancy == ENOMR_OCCUPANCY_HIGH || list) return false;
+    if (c->occupancy == ENOMR_OCCUPANCY_HIGH) return false;
     const long long tiles = ((c->nx + X_TP - 2) / (X_TP - 1)) * ((c->ny + X_NL - 1) / X_NL);
-    return tiles < 4LL * c->sms * (SWEEP_HIGH_THREADS_PER_SM / (X_TP * X_NL));
+    const long long wave = c->sms * (SWEEP_HIGH_THREADS_PER_SM / (X_TP * X_NL));
+    return list ? 4 * tiles < 7 * wave : tiles < 4 * wave;
 }
 
 // Evaluate L(U) into the epilogue.  The alpha of U must be current.
