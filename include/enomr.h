@@ -27,6 +27,10 @@
  *           (rho <= 0, p <= 0, Roe c^2 <= 0, NaN/Inf) set a device status
  *           word that enomr_get_status() reads; the kernels never trap,
  *           abort or print.
+ * Scale.    Units do not matter to the results, beyond rounding, but to the time:
+ *           windows whose differences lie below 2^-60 or values above 2^90 are
+ *           selected in FP64 alone (smooth lines: about twice the time of the
+ *           float form, random ones up to eight times).
  * Grid.     Uniform spacing dx (dy).  Boundary: periodic (requires
  *           nx, ny >= 2g, g = (order+1)/2) or transmissive (zeroth-order
  *           extrapolation into g ghost cells).

@@ -61,10 +61,13 @@ constexpr int LONG_TAIL = 16;
 // cells are already in shared memory (the TMA ring of enomr_tma.cuh) reads
 // them in place.
 // kFloatSelect: selections by mr_select, else by mr_select64: with boundary
-// sides, whose flows leave most of the grid constant up to rounding (the wake
-// of the double Mach reflection: 94 % of the windows end in S(0,0)), the float
-// form is left open nearly everywhere and only adds its differences (y sweep,
-// 1200 x 300 after 300 steps: 541 against 513 us).
+// sides or a body force.  The wake of the double Mach reflection is constant up
+// to rounding (94 % of its windows end in S(0,0)), and on grids of few tiles the
+// float form adds its latency: a step with mr_select64 / mr_select, 300 x 75 after
+// 20 steps, order 5, 9, 17: 340 / 355, 499 / 552, 1134 / 1288 us; 1200 x 300 after
+// 100 steps 915 / 912, 1309 / 1282, 2762 / 2653.  Larger grids and flows without
+// such regions would gain (2400 x 600 2 to 9 %; 512^2 random cells with a force,
+// order 9, 3.7 / 1.9 ms).
 template <int R, int C, int DIR, int TP, int NL, bool FS = true>
 struct ClassicTile {
     static constexpr bool kFloatSelect = FS;

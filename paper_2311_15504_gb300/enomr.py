@@ -294,8 +294,8 @@ class Solver:
             self.set_side(i, sd[0], sd[1], sd[2], sd[3], sd[4], sd[5])
 
     def set_staging(self, mode):
-        """STAGING_AUTO (TMA where the state allows it), STAGING_LOADS or
-        STAGING_TMA (TMA only; other states raise)."""
+        """STAGING_AUTO (plain loads over tile lists, else TMA where the state
+        allows it), STAGING_LOADS or STAGING_TMA (TMA only; other states raise)."""
         _check(_lib.enomr_set_staging(self._ctx, int(mode)), "enomr_set_staging")
 
     def set_occupancy(self, mode):

@@ -6,7 +6,8 @@ cover tiles at both ends of the lines (ghosts filled after the copy),
 ragged last tiles, line counts that are not a multiple of the tile's lines
 (rows or columns past the grid), lines shorter than one tile, both boundary
 types and every order; the CUDA path's agreement with the oracle is checked
-by the parity tests, which take the TMA path wherever nx is even.
+by the parity tests, which take the TMA path on grids below 2^16 cells with nx
+even.
 """
 import numpy as np
 import pytest
