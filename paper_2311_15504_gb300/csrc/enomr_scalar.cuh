@@ -275,10 +275,10 @@ namespace enomr {
 // open is spread as in their launches.  A line of n <= SMALL_CELLS is a few warps
 // of work; launched one stage at a time it costs four (Burgers: seven) launches
 // of about 5 us each.  A step, by launches of one stage each / in one CTA / over a
-// cluster: advection, order 5, 200 cells 23.7 / 15.7 / 15.8 us; 1024 cells, smooth
-// 23.8 / 21.5 / 14.1, constant up to rounding 27 / 58 / 20; order 17, random cells
-// 92 / 56 / 20, constant up to rounding 92 / 325 / 77; Burgers, order 9, smooth
-// 43 / 25 / 16.
+// cluster: advection, order 5, 1024 cells, smooth 23.8 / 21.5 / 14.1 us, constant
+// up to rounding 27 / 58 / 20; order 17, random cells 92 / 56 / 20, constant up to
+// rounding 92 / 325 / 77; Burgers, order 9, smooth 43 / 25 / 16; 200 cells, one CTA,
+// order 5, bound by the host: 23.7 / 15.7 / 15.8, on the device alone - / 7.4 / 7.1.
 // ---------------------------------------------------------------------------
 template <int R, bool BURGERS>
 struct SmallSmem {
@@ -425,7 +425,7 @@ template <int R> cudaError_t launch_scalar_step(const SmallArgs &a, bool burgers
     cfg.blockDim = dim3(SMALL_THREADS);
     cfg.stream = s;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = a.n > SMALL_TILE ? 1 : 0;  // one CTA: 0.5 us less than as a cluster of one
     return burgers ? cudaLaunchKernelEx(&cfg, k_scalar_step<R, true>, a)
                    : cudaLaunchKernelEx(&cfg, k_scalar_step<R, false>, a);
 }
